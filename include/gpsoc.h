@@ -373,7 +373,7 @@ gpsoc_status gpsoc_probe_peaks(double* fp64_tflops, double* fp32_tflops);
  *   obs:    host, 9 doubles per solve as gpsoc_apply_h (may be NULL);
  *   cuda_stream: cudaStream_t or NULL (legacy default stream); the call
  *           returns after the stream has finished its work.
- * It allocates nothing: intermediate arrays, partial sums, twiddle tables and
+ * It allocates nothing: intermediate arrays, partial sums and
  * per-solve scalars live in one fixed 16 MiB array in device memory, present on
  * every GPU that loads the library until the process exits.  The first call on
  * a device looks up the array's device address (cudaGetSymbolAddress) and sets

@@ -33,45 +33,31 @@ static constexpr int kRedDoubles = 16 * (kThreads / 32) + 16;
 // entry (r, j) = W_n^(r j), r < E, j < n/E, at the padded index fft_pad(r n/E + j).
 // The last pass (radix E, Ns = n/E) reads j = k for consecutive groups k:
 // consecutive addresses; earlier passes read j = k n/(Ns E) for few distinct k.
+// FP64 passes transform in fixed point (fixfft.cuh) with a table of their own.
 template <class T>
 __device__ __forceinline__ void load_tw(cx_t<T>* s_tw, const cx_t<T>* tw, int n, int ept) {
-  const int lc = __ffs(n / ept) - 1;   // log2(n / E): n and E are powers of two
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const int r = i >> lc, j = i & ((1 << lc) - 1);
-    s_tw[fft_pad<cx_t<T>>(i)] = tw[r * j];
-  }
-}
-
-// Row tiles: nlines lines of padded length NP; thread -> (line q, group g0), E
-// elements per thread.  NI = 2 transforms the same line of buf0 and buf1 together.
-template <class C, bool INV, int NI, int E>
-__device__ __forceinline__ void row_fft_e(C* buf0, C* buf1, int nlines, int NP, int L, const C* tw) {
-  const int G = (1 << L) / E;
-  const int q = threadIdx.x / G, g0 = threadIdx.x - q * G;
-  const bool act = q < nlines;
-  const int qq = act ? q : 0;
-  if constexpr (NI == 2) {
-    C* const l2[2] = {buf0 + qq * NP, buf1 + qq * NP};
-    const bool a2[2] = {act, act};
-    stockham_fft<C, INV, E, 2>(l2, a2, g0, 1, L, tw);
+  if constexpr (sizeof(T) == 8) {
+    fx_load_tw(reinterpret_cast<FxW*>(s_tw), n, ept == 8 ? 8 : 4, FftPad16{});
   } else {
-    C* const l1[1] = {buf0 + qq * NP};
-    const bool a1[1] = {act};
-    stockham_fft<C, INV, E, 1>(l1, a1, g0, 1, L, tw);
+    const int lc = __ffs(n / ept) - 1;   // log2(n / E): n and E are powers of two
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const int r = i >> lc, j = i & ((1 << lc) - 1);
+      s_tw[fft_pad<cx_t<T>>(i)] = tw[r * j];
+    }
   }
 }
 
-// R16: the kernel may run radix-16 passes (FP32 column passes only: the code path
-// sets the register allocation of the whole kernel, and FP64 or two-line row
-// tiles would lose occupancy to it)
-template <class C, bool INV, int NI, bool R16 = false>
-__device__ __forceinline__ void row_fft(C* buf0, C* buf1, int nlines, int NP, int L, const C* tw, int ept) {
+// transforms of nlines lines at offset off (see fft_lines_e).  R16: the kernel may run radix-16 passes
+// (FP32 column passes only: the code path sets the register allocation of the whole kernel).
+// FP64 tiles of 2 elements per thread transform with half their threads.
+template <class C, bool R16 = false>
+__device__ __forceinline__ void fft_lines(int off, int nlines, int NP, int L, int ept) {
   if constexpr (R16 && sizeof(C) == 8) {
-    if (ept == 16) { row_fft_e<C, INV, NI, 16>(buf0, buf1, nlines, NP, L, tw); return; }
+    if (ept == 16) { fft_lines_e<C, 16>(off, nlines, NP, L); return; }
   }
-  if (ept == 8) row_fft_e<C, INV, NI, 8>(buf0, buf1, nlines, NP, L, tw);
-  else if (ept == 4) row_fft_e<C, INV, NI, 4>(buf0, buf1, nlines, NP, L, tw);
-  else row_fft_e<C, INV, NI, 2>(buf0, buf1, nlines, NP, L, tw);
+  if (ept == 8) fft_lines_e<C, 8>(off, nlines, NP, L);
+  else if (ept == 4 || sizeof(C) == 16) fft_lines_e<C, 4>(off, nlines, NP, L);
+  else if constexpr (sizeof(C) == 8) fft_lines_e<C, 2>(off, nlines, NP, L);
 }
 
 // padded length of a column line in shared memory
@@ -137,7 +123,8 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
   load_tw<T>(s_tw, A.tw[0], nx, ept);   // constant table: before the wait on the previous kernel
   pdl_wait();
   if (s >= A.nsolve || !gate_ok(A.st, A.gate, s)) return;
-  C* buf0 = s_tw + fft_padded_len<C>(nx);
+  const int b0 = fft_padded_len<C>(nx);   // the lines lie behind the table
+  C* buf0 = s_tw + b0;
   const int per = R * nx;             // elements of one component in the tile
   const int NP = fft_padded_len<C>(nx), CP = R * NP;   // padded line length, component stride in smem
   constexpr bool two = (MODE == ROW_INV_H || MODE == ROW_INV_P || MODE == ROW_INV_LIN || MODE == ROW_INV_P_HY);
@@ -254,7 +241,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
       }
     }
     __syncthreads();
-    row_fft<C, false, 1>(buf0, buf1, 3 * R, NP, Lx, s_tw, ept);
+    fft_lines<C>(b0, 3 * R, NP, Lx, ept);
     for (int e = threadIdx.x; e < per; e += blockDim.x) {
       const int pos = (e / nx) * NP + fft_pad<C>(e % nx);
 #pragma unroll
@@ -272,18 +259,17 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
   }
 
   // ---------------------------------------------------------------- inverse passes
-  // natural order in shared memory, inverse transform in place
+  // natural order in shared memory, inverse transform in place (both arrays' lines in one call)
   for (int e = threadIdx.x; e < per; e += blockDim.x) {
     const int pos = (e / nx) * NP + fft_pad<C>(e % nx);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      buf0[c * CP + pos] = A.in0[sbase + c * npts + rbase + e];
-      if (two) buf1[c * CP + pos] = A.in1[sbase + c * npts + rbase + e];
+      buf0[c * CP + pos] = swp(A.in0[sbase + c * npts + rbase + e]);
+      if (two) buf1[c * CP + pos] = swp(A.in1[sbase + c * npts + rbase + e]);
     }
   }
   __syncthreads();
-  if (two) row_fft<C, true, 2>(buf0, buf1, 3 * R, NP, Lx, s_tw, ept);
-  else row_fft<C, true, 1>(buf0, buf1, 3 * R, NP, Lx, s_tw, ept);
+  fft_lines<C>(b0, two ? 6 * R : 3 * R, NP, Lx, ept);
 
   const W inv_n = (W)1 / (W)npts;
   const W Om = pick<W>(ph.Omega, ph.fOmega);
@@ -294,7 +280,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
       const int pos = r * NP + fft_pad<C>(j);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const C v = buf0[c * CP + pos];
+        const C v = swp(buf0[c * CP + pos]);
         A.out0[sbase + c * npts + rbase + e] = mk<C>(v.x * sc, v.y * sc);
       }
     }
@@ -327,7 +313,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
         W den = al[c] + V + c0 * rho;
         den = fmax(den, (W)1e-12 * al[c]);
         const W sc = use_pv ? inv_n * rsqrt_w<W>(den) : inv_n;
-        const C v = buf0[c * CP + pos];
+        const C v = swp(buf0[c * CP + pos]);
         const C z = mk<C>(v.x * sc, v.y * sc);
         A.out0[sbase + c * npts + off] = z;
         const C rr = A.in2[sbase + c * npts + off];
@@ -368,8 +354,8 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       u[c] = A.in2[sbase + c * npts + off];
-      const C t = buf0[c * CP + pos];
-      const C gg = buf1[c * CP + pos];
+      const C t = swp(buf0[c * CP + pos]);
+      const C gg = swp(buf1[c * CP + pos]);
       lin_r[c] = (t.x - Om * x * gg.x) * inv_n + V * u[c].x;
       lin_i[c] = (t.y - Om * x * gg.y) * inv_n + V * u[c].y;
     }
@@ -532,7 +518,8 @@ __global__ void __launch_bounds__(kThreads) k_col(ChainArgs<T> A, int axis, int 
   if (s >= A.nsolve || !gate_ok(A.st, A.gate, s)) return;
   const int o = tb / tpo;
   const int i0 = (tb % tpo) * TC;
-  C* buf = s_tw + fft_padded_len<C>(na);
+  const int b0 = fft_padded_len<C>(na);   // the lines lie behind the table
+  C* buf = s_tw + b0;
   const int per = na * TC;
   const int NPL = col_line_len<C>(na, TC);        // padded line length
   const int CS = TC * NPL;                     // component stride in smem
@@ -552,34 +539,12 @@ __global__ void __launch_bounds__(kThreads) k_col(ChainArgs<T> A, int axis, int 
     const int j = e / TC, t = e - j * TC;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      buf[sidx(c, t, j)] = A.in0[sbase + c * npts + obase + (long long)j * ni + t];
+      const C v = A.in0[sbase + c * npts + obase + (long long)j * ni + t];
+      buf[sidx(c, t, j)] = (MODE == COL_INV || MODE == COL_YINV_H) ? swp(v) : v;
       if (MODE == COL_YINV_H) buf2[sidx(c, t, j)] = A.in1[sbase + c * npts + obase + (long long)j * ni + t];
     }
   }
   __syncthreads();
-
-  if (MODE == COL_FWD) {
-    row_fft<C, false, 1, true>(buf, buf, 3 * TC, NPL, La, s_tw, ept);
-    for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int j = e / TC, t = e - j * TC;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) A.out0[sbase + c * npts + obase + (long long)j * ni + t] = buf[sidx(c, t, j)];
-    }
-    return;
-  }
-  if (MODE == COL_INV) {
-    row_fft<C, true, 1, true>(buf, buf, 3 * TC, NPL, La, s_tw, ept);
-    const W sc = (W)A.scale;
-    for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int j = e / TC, t = e - j * TC;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const C v = buf[sidx(c, t, j)];
-        A.out0[sbase + c * npts + obase + (long long)j * ni + t] = mk<C>(v.x * sc, v.y * sc);
-      }
-    }
-    return;
-  }
 
   // inner index -> (kx [, ky]) wavenumbers (inputs are spectral along the faster axes)
   auto kinner = [&](int t, W& kx, W& ky) {
@@ -588,18 +553,139 @@ __global__ void __launch_bounds__(kThreads) k_col(ChainArgs<T> A, int axis, int 
     else { kx = wavenum<W>(ii % nx, nx, geo_piL<W>(A.g, 0)); ky = wavenum<W>(ii / nx, A.g.n[1], geo_piL<W>(A.g, 1)); }
   };
 
-  if (MODE == COL_YINV_H) {
-    // buf: C -> F_y^-1 C;  buf2: A -> F_y A, times v_y, F_y^-1 -> G
-    row_fft<C, true, 1, true>(buf, buf, 3 * TC, NPL, La, s_tw, ept);
-    row_fft<C, false, 1, true>(buf2, buf2, 3 * TC, NPL, La, s_tw, ept);
+  W acc[3] = {(W)0, (W)0, (W)0};
+  // one transform, or (the middle passes) a forward one, the work in k and the inverse one: a loop
+  // around one inlined copy of the transforms
+  constexpr bool middle = (MODE == COL_MID_H || MODE == COL_MID_PRE || MODE == COL_YMID_H || MODE == COL_YINV_H);
+#pragma unroll 1
+  for (int phase = 0; phase < (middle ? 2 : 1); ++phase) {
+    if (MODE == COL_YINV_H && phase == 1) {
+      // buf2: A -> F_y A, times v_y; then F_y^-1 of both: buf from C, buf2 -> G
+      for (int e = threadIdx.x; e < per; e += blockDim.x) {
+        const int j = e / TC, t = e - j * TC;
+        const W vy = wavenum<W>(j, na, piA);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) buf2[sidx(c, t, j)] = swp(cscale(buf2[sidx(c, t, j)], vy));
+      }
+      __syncthreads();
+    } else if (phase == 1) {
+      if (sizeof(T) == 4 && (MODE == COL_YMID_H || MODE == COL_MID_H) && A.xhat) {
+        // GPSOC_HYBRID P chain: buf holds the full spectrum of P.  Advance the stored spectrum
+        // of Phi by the step applied this iteration (Phi_hat <- g (c Phi_hat + t P_hat_prev)),
+        // keep this P_hat, and sum 1/2 |k|^2 |Phi_hat_l|^2 and 1/2 |k|^2 Re(Phi_hat_l conj P_hat_l)
+        const bool upd = A.khat_upd && S.upd_applied;
+        const W uc = pick<W>(S.upd_c, S.fupd_c), us = pick<W>(S.upd_s, S.fupd_s), usc = pick<W>(S.upd_scale, S.fupd_scale);
+        W kacc[6] = {(W)0, (W)0, (W)0, (W)0, (W)0, (W)0};
+        for (int e = threadIdx.x; e < per; e += blockDim.x) {
+          const int j = e / TC, t = e - j * TC;
+          W kx, ky, kz = (W)0;
+          kinner(t, kx, ky);
+          if (axis == 1) ky = wavenum<W>(j, na, piA);
+          else kz = wavenum<W>(j, na, piA);
+          const W k2h = (W)0.5 * (kx * kx + ky * ky + kz * kz);
+          const long long gi = sbase + obase + (long long)j * ni + t;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const C pv = buf[sidx(c, t, j)];
+            C xv = A.xhat[gi + c * npts];
+            if (upd) {
+              const C po = A.phat[gi + c * npts];
+              xv = mk<C>(usc * (uc * xv.x + us * po.x), usc * (uc * xv.y + us * po.y));
+              A.xhat[gi + c * npts] = xv;
+            }
+            A.phat[gi + c * npts] = pv;
+            kacc[c] += k2h * (xv.x * xv.x + xv.y * xv.y);
+            kacc[3 + c] += k2h * (xv.x * pv.x + xv.y * pv.y);
+          }
+        }
+        const bool kmx[6] = {false, false, false, false, false, false};
+        const int kslots[6] = {SL_KPHI0, SL_KPHI1, SL_KPHI2, SL_KX0, SL_KX1, SL_KX2};
+        store_partials<6, W>(kacc, kslots, kmx, red, A.part, (long long)s * NSLOT, A.pmax, tb);
+      }
+
+      // pointwise in k: the kinetic + SOC symbol (H chains) or the kinetic preconditioner; with
+      // YMID_H also G_c = F_y^-1[v_y F_y A_c] in buf2.  Results go back exchanged (inverse transform)
+      const W al[3] = {pick<W>(S.alpha[0], S.falpha[0]), pick<W>(S.alpha[1], S.falpha[1]), pick<W>(S.alpha[2], S.falpha[2])};
+      const W g = pick<W>(ph.gamma, ph.fgamma);
+      const bool use_pd = (A.sc.opts.precond == GPSOC_PRECOND_COMBINED || A.sc.opts.precond == GPSOC_PRECOND_KINETIC);
+      for (int e = threadIdx.x; e < per; e += blockDim.x) {
+        const int j = e / TC, t = e - j * TC;
+        const int i1 = sidx(0, t, j), i2 = sidx(1, t, j), i3 = sidx(2, t, j);
+        W kx, ky, kz = (W)0;
+        kinner(t, kx, ky);
+        if (axis == 1) ky = wavenum<W>(j, na, piA);
+        else kz = wavenum<W>(j, na, piA);
+        const W k2h = (W)0.5 * (kx * kx + ky * ky + kz * kz);
+        if (MODE == COL_MID_PRE) {
+          // P_Delta (Eq. PreCondKin); the potential-only and no-preconditioner variants keep
+          // the coefficients (the transform pair is then the identity up to rounding)
+          if (use_pd) {
+            // the three reciprocals from one division (an FP64 division is a long
+            // instruction sequence): 1/d0 = d1 d2 / (d0 d1 d2), and so on
+            const W d0 = al[0] + k2h, d1 = al[1] + k2h, d2 = al[2] + k2h;
+            const W d01 = d0 * d1;
+            const W inv = (W)1 / (d01 * d2);
+            const W r01 = d2 * inv;
+            buf[i1] = swp(cscale(buf[i1], d1 * r01));
+            buf[i2] = swp(cscale(buf[i2], d0 * r01));
+            buf[i3] = swp(cscale(buf[i3], d01 * inv));
+          } else {
+            buf[i1] = swp(buf[i1]);
+            buf[i2] = swp(buf[i2]);
+            buf[i3] = swp(buf[i3]);
+          }
+        } else {
+          const C p1 = buf[i1], p0 = buf[i2], pm = buf[i3];
+          if (MODE == COL_YMID_H) {
+            buf2[i1] = swp(cscale(p1, ky));
+            buf2[i2] = swp(cscale(p0, ky));
+            buf2[i3] = swp(cscale(pm, ky));
+          }
+          // kinetic per component (Parseval): sum 1/2 |k|^2 |phat_l|^2
+          acc[0] += k2h * (p1.x * p1.x + p1.y * p1.y);
+          acc[1] += k2h * (p0.x * p0.x + p0.y * p0.y);
+          acc[2] += k2h * (pm.x * pm.x + pm.y * pm.y);
+          // -gamma S symbol: s0 = -kx + i ky (L0), s1 = -(kx + i ky) (L1)
+          // out_1 = K p1 - g s0 p0 ; out_0 = K p0 - g (s1 p1 + s0 pm) ; out_-1 = K pm - g s1 p0
+          const W s0r = -kx, s0i = ky, s1r = -kx, s1i = -ky;
+          const W a_r = s0r * p0.x - s0i * p0.y, a_i = s0r * p0.y + s0i * p0.x;   // s0 p0
+          const W b_r = s1r * p1.x - s1i * p1.y, b_i = s1r * p1.y + s1i * p1.x;   // s1 p1
+          const W c_r = s0r * pm.x - s0i * pm.y, c_i = s0r * pm.y + s0i * pm.x;   // s0 pm
+          const W d_r = s1r * p0.x - s1i * p0.y, d_i = s1r * p0.y + s1i * p0.x;   // s1 p0
+          buf[i1] = mk<C>(k2h * p1.y - g * a_i, k2h * p1.x - g * a_r);
+          buf[i2] = mk<C>(k2h * p0.y - g * (b_i + c_i), k2h * p0.x - g * (b_r + c_r));
+          buf[i3] = mk<C>(k2h * pm.y - g * d_i, k2h * pm.x - g * d_r);
+        }
+      }
+      __syncthreads();
+    }
+    int first = b0, lines = 3 * TC;
+    if (MODE == COL_YINV_H && phase == 0) first = b0 + 3 * CS;
+    if ((MODE == COL_YINV_H || MODE == COL_YMID_H) && phase == 1) lines = 6 * TC;
+    fft_lines<C, true>(first, lines, NPL, La, ept);
+  }
+
+  if (MODE == COL_FWD) {
     for (int e = threadIdx.x; e < per; e += blockDim.x) {
       const int j = e / TC, t = e - j * TC;
-      const W vy = wavenum<W>(j, na, piA);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) buf2[sidx(c, t, j)] = cscale(buf2[sidx(c, t, j)], vy);
+      for (int c = 0; c < 3; ++c) A.out0[sbase + c * npts + obase + (long long)j * ni + t] = buf[sidx(c, t, j)];
     }
-    __syncthreads();
-    row_fft<C, true, 1, true>(buf2, buf2, 3 * TC, NPL, La, s_tw, ept);
+    return;
+  }
+  if (MODE == COL_INV) {
+    const W sc = (W)A.scale;
+    for (int e = threadIdx.x; e < per; e += blockDim.x) {
+      const int j = e / TC, t = e - j * TC;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const C v = swp(buf[sidx(c, t, j)]);
+        A.out0[sbase + c * npts + obase + (long long)j * ni + t] = mk<C>(v.x * sc, v.y * sc);
+      }
+    }
+    return;
+  }
+  if (MODE == COL_YINV_H) {
     const W nfac = (W)A.g.n[1] * (W)A.g.n[2];  // ny * nz
     const W nz = (W)A.g.n[2];
     for (int e = threadIdx.x; e < per; e += blockDim.x) {
@@ -612,116 +698,14 @@ __global__ void __launch_bounds__(kThreads) k_col(ChainArgs<T> A, int axis, int 
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const C a = A.in1[gi + c * npts];
-        const C cv = buf[sidx(c, t, j)];
+        const C cv = swp(buf[sidx(c, t, j)]);
         A.out0[gi + c * npts] = mk<C>(cv.x + rot * a.x, cv.y + rot * a.y);
-        const C gv = buf2[sidx(c, t, j)];
+        const C gv = swp(buf2[sidx(c, t, j)]);
         A.out1[gi + c * npts] = mk<C>(gv.x * nz, gv.y * nz);
       }
     }
     return;
   }
-
-  // forward transform along the axis: natural-order spectrum in buf
-  row_fft<C, false, 1, true>(buf, buf, 3 * TC, NPL, La, s_tw, ept);
-
-  if ((MODE == COL_YMID_H || MODE == COL_MID_H) && A.xhat) {
-    // GPSOC_HYBRID P chain: buf holds the full spectrum of P.  Advance the stored spectrum
-    // of Phi by the step applied this iteration (Phi_hat <- g (c Phi_hat + t P_hat_prev)),
-    // keep this P_hat, and sum 1/2 |k|^2 |Phi_hat_l|^2 and 1/2 |k|^2 Re(Phi_hat_l conj P_hat_l)
-    const bool upd = A.khat_upd && S.upd_applied;
-    const W uc = pick<W>(S.upd_c, S.fupd_c), us = pick<W>(S.upd_s, S.fupd_s), usc = pick<W>(S.upd_scale, S.fupd_scale);
-    W kacc[6] = {(W)0, (W)0, (W)0, (W)0, (W)0, (W)0};
-    for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int j = e / TC, t = e - j * TC;
-      W kx, ky, kz = (W)0;
-      kinner(t, kx, ky);
-      if (axis == 1) ky = wavenum<W>(j, na, piA);
-      else kz = wavenum<W>(j, na, piA);
-      const W k2h = (W)0.5 * (kx * kx + ky * ky + kz * kz);
-      const long long gi = sbase + obase + (long long)j * ni + t;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const C pv = buf[sidx(c, t, j)];
-        C xv = A.xhat[gi + c * npts];
-        if (upd) {
-          const C po = A.phat[gi + c * npts];
-          xv = mk<C>(usc * (uc * xv.x + us * po.x), usc * (uc * xv.y + us * po.y));
-          A.xhat[gi + c * npts] = xv;
-        }
-        A.phat[gi + c * npts] = pv;
-        kacc[c] += k2h * (xv.x * xv.x + xv.y * xv.y);
-        kacc[3 + c] += k2h * (xv.x * pv.x + xv.y * pv.y);
-      }
-    }
-    const bool kmx[6] = {false, false, false, false, false, false};
-    const int kslots[6] = {SL_KPHI0, SL_KPHI1, SL_KPHI2, SL_KX0, SL_KX1, SL_KX2};
-    store_partials<6, W>(kacc, kslots, kmx, red, A.part, (long long)s * NSLOT, A.pmax, tb);
-  }
-
-  if (MODE == COL_YMID_H) {
-    // G_c = F_y^-1[v_y F_y A_c] for the three components at once (buf2)
-    for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int j = e / TC, t = e - j * TC;
-      const W vy = wavenum<W>(j, na, piA);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) buf2[sidx(c, t, j)] = cscale(buf[sidx(c, t, j)], vy);
-    }
-    __syncthreads();
-    row_fft<C, true, 1, true>(buf2, buf2, 3 * TC, NPL, La, s_tw, ept);
-    for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int j = e / TC, t = e - j * TC;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) A.out1[sbase + c * npts + obase + (long long)j * ni + t] = buf2[sidx(c, t, j)];
-    }
-  }
-
-  W acc[3] = {(W)0, (W)0, (W)0};
-  // pointwise in k: the kinetic + SOC symbol (H chains) or the kinetic preconditioner
-  const W al[3] = {pick<W>(S.alpha[0], S.falpha[0]), pick<W>(S.alpha[1], S.falpha[1]), pick<W>(S.alpha[2], S.falpha[2])};
-  const W g = pick<W>(ph.gamma, ph.fgamma);
-  const bool use_pd = (A.sc.opts.precond == GPSOC_PRECOND_COMBINED || A.sc.opts.precond == GPSOC_PRECOND_KINETIC);
-  for (int e = threadIdx.x; e < per; e += blockDim.x) {
-    const int j = e / TC, t = e - j * TC;
-    const int i1 = sidx(0, t, j), i2 = sidx(1, t, j), i3 = sidx(2, t, j);
-    W kx, ky, kz = (W)0;
-    kinner(t, kx, ky);
-    if (axis == 1) ky = wavenum<W>(j, na, piA);
-    else kz = wavenum<W>(j, na, piA);
-    const W k2h = (W)0.5 * (kx * kx + ky * ky + kz * kz);
-    if (MODE == COL_MID_PRE) {
-      // P_Delta (Eq. PreCondKin); the potential-only and no-preconditioner variants keep
-      // the coefficients (the transform pair is then the identity up to rounding)
-      if (use_pd) {
-        // the three reciprocals from one division (an FP64 division is a long
-        // instruction sequence): 1/d0 = d1 d2 / (d0 d1 d2), and so on
-        const W d0 = al[0] + k2h, d1 = al[1] + k2h, d2 = al[2] + k2h;
-        const W d01 = d0 * d1;
-        const W inv = (W)1 / (d01 * d2);
-        const W r01 = d2 * inv;
-        buf[i1] = cscale(buf[i1], d1 * r01);
-        buf[i2] = cscale(buf[i2], d0 * r01);
-        buf[i3] = cscale(buf[i3], d01 * inv);
-      }
-    } else {
-      const C p1 = buf[i1], p0 = buf[i2], pm = buf[i3];
-      // kinetic per component (Parseval): sum 1/2 |k|^2 |phat_l|^2
-      acc[0] += k2h * (p1.x * p1.x + p1.y * p1.y);
-      acc[1] += k2h * (p0.x * p0.x + p0.y * p0.y);
-      acc[2] += k2h * (pm.x * pm.x + pm.y * pm.y);
-      // -gamma S symbol: s0 = -kx + i ky (L0), s1 = -(kx + i ky) (L1)
-      // out_1 = K p1 - g s0 p0 ; out_0 = K p0 - g (s1 p1 + s0 pm) ; out_-1 = K pm - g s1 p0
-      const W s0r = -kx, s0i = ky, s1r = -kx, s1i = -ky;
-      const W a_r = s0r * p0.x - s0i * p0.y, a_i = s0r * p0.y + s0i * p0.x;   // s0 p0
-      const W b_r = s1r * p1.x - s1i * p1.y, b_i = s1r * p1.y + s1i * p1.x;   // s1 p1
-      const W c_r = s0r * pm.x - s0i * pm.y, c_i = s0r * pm.y + s0i * pm.x;   // s0 pm
-      const W d_r = s1r * p0.x - s1i * p0.y, d_i = s1r * p0.y + s1i * p0.x;   // s1 p0
-      buf[i1] = mk<C>(k2h * p1.x - g * a_r, k2h * p1.y - g * a_i);
-      buf[i2] = mk<C>(k2h * p0.x - g * (b_r + c_r), k2h * p0.y - g * (b_i + c_i));
-      buf[i3] = mk<C>(k2h * pm.x - g * d_r, k2h * pm.y - g * d_i);
-    }
-  }
-  __syncthreads();
-  row_fft<C, true, 1, true>(buf, buf, 3 * TC, NPL, La, s_tw, ept);
 
   const W nrot = (W)A.g.n[1];  // 2D: T' = F_y^-1[M F_y A] + ny Omega y v_x A
   const W Om = pick<W>(ph.Omega, ph.fOmega);
@@ -736,12 +720,13 @@ __global__ void __launch_bounds__(kThreads) k_col(ChainArgs<T> A, int axis, int 
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const C a = A.in0[gi + c * npts];
-        const C v = buf[sidx(c, t, j)];
+        const C v = swp(buf[sidx(c, t, j)]);
         A.out0[gi + c * npts] = mk<C>(v.x + rot * a.x, v.y + rot * a.y);
+        A.out1[gi + c * npts] = swp(buf2[sidx(c, t, j)]);
       }
     } else {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) A.out0[gi + c * npts] = buf[sidx(c, t, j)];
+      for (int c = 0; c < 3; ++c) A.out0[gi + c * npts] = swp(buf[sidx(c, t, j)]);
     }
   }
   if (MODE == COL_MID_H || MODE == COL_YMID_H) {

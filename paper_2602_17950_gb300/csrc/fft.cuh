@@ -17,6 +17,7 @@
 // fft_pad(r N/E + j) (E = elements per thread, the radix of the last pass).
 #pragma once
 
+#include "fixfft.cuh"
 #include "gpsoc_internal.cuh"
 
 namespace gpsoc {
@@ -26,11 +27,6 @@ namespace gpsoc {
 template <class C> constexpr int kPadShift = (sizeof(C) == 8) ? 4 : 3;
 template <class C> __host__ __device__ __forceinline__ int fft_pad(int e) { return e + (e >> kPadShift<C>); }
 template <class C> __host__ __device__ __forceinline__ int fft_padded_len(int n) { return n + (n >> kPadShift<C>); }
-
-template <class C> __device__ __forceinline__ C cmul_conj_if(C a, C w, bool conj) {
-  if (conj) w.y = -w.y;
-  return cmul(a, w);
-}
 
 // multiply by -i (forward) or +i (inverse)
 template <class C, bool INV> __device__ __forceinline__ C mul_mi(C a) {
@@ -141,71 +137,108 @@ template <class C, bool INV, int R, int E> __device__ __forceinline__ void dftR(
   }
 }
 
-// One Stockham pass of radix R for NI work items per thread holding E elements
-// each (E >= R).  Item it of this thread covers line lines[it] (element stride
-// es, padded indices) and the E/R groups g0 + u N/E (u < E/R).  Inactive items
-// only take part in the barriers.
-template <class C, bool INV, int R, int E, int NI>
-__device__ __forceinline__ void stockham_pass(C* const (&lines)[NI], const bool (&active)[NI], int g0, int es, int N,
-                                              int Ns, const C* tw) {
-  constexpr int PER = E / R;   // radix-R groups handled by one item
-  C v[NI][E];
+// One Stockham pass of radix R over the line at p, E elements per thread (E >= R): this thread's
+// E/R groups are g0 + u N/E (u < E/R).  Inactive threads only synchronise.
+template <class C, int R, int E>
+__device__ __forceinline__ void stockham_pass(C* p, bool act, int g0, int N, int Ns, const C* tw, bool warp) {
+  constexpr int PER = E / R;   // radix-R groups of one thread
+  C v[E];
   const int NR = N / R;
-#pragma unroll
-  for (int it = 0; it < NI; ++it) {
-    if (!active[it]) continue;
+  if (act) {
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
       const int g = g0 + u * (N / E);
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[it][u * R + r] = lines[it][fft_pad<C>(g + r * NR) * es];
+      for (int r = 0; r < R; ++r) v[u * R + r] = p[fft_pad<C>(g + r * NR)];
     }
-  }
-  __syncthreads();
+  } else {
 #pragma unroll
-  for (int it = 0; it < NI; ++it) {
-    if (!active[it]) continue;
+    for (int e = 0; e < E; ++e) v[e] = mk<C>(0.0f, 0.0f);   // as in fx_pass
+  }
+  fx_sync(warp);
+  if (act) {
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
       const int g = g0 + u * (N / E);
-      const int k = g % Ns;
+      const int k = g & (Ns - 1);
       if (k != 0) {
         // W_N^(r k N / (Ns R)): entry (r, k N / (Ns R)) of the table (R = E here:
         // only the first pass, with k = 0, can have a smaller radix)
         const int j = k * (N / (Ns * R));
 #pragma unroll
-        for (int r = 1; r < R; ++r)
-          v[it][u * R + r] = cmul_conj_if(v[it][u * R + r], tw[fft_pad<C>(r * (N / E) + j)], INV);
+        for (int r = 1; r < R; ++r) v[u * R + r] = cmul(v[u * R + r], tw[fft_pad<C>(r * (N / E) + j)]);
       }
-      dftR<C, INV, R, E>(v[it], u * R);
-      const int ob = (g / Ns) * Ns * R + k;
+      dftR<C, false, R, E>(v, u * R);
+      const int ob = (g - k) * R + k;
 #pragma unroll
-      for (int q = 0; q < R; ++q) lines[it][fft_pad<C>(ob + q * Ns) * es] = v[it][u * R + q];
+      for (int q = 0; q < R; ++q) p[fft_pad<C>(ob + q * Ns)] = v[u * R + q];
     }
+  }
+  fx_sync(warp);
+}
+
+// The transform of length N = 2^L (N >= E) of one line per N/E threads (E in {2, 4, 8, 16}:
+// radix-E passes plus one smaller pass when log2 N is not a multiple of log2 E).
+template <class C, int E>
+__device__ __forceinline__ void stockham_fft(C* p, bool act, int g0, int L, const C* tw, bool warp) {
+  const int N = 1 << L;
+  int Ns = 1;
+  constexpr int LE = (E == 16) ? 4 : (E == 8) ? 3 : (E == 4) ? 2 : 1;
+  const int rem = L % LE;
+  if (rem == 1) { stockham_pass<C, 2, E>(p, act, g0, N, Ns, tw, warp); Ns *= 2; }
+  else if (rem == 2) { if constexpr (E >= 4) { stockham_pass<C, 4, E>(p, act, g0, N, Ns, tw, warp); Ns *= 4; } }
+  else if constexpr (E == 16) {
+    if (rem == 3) { stockham_pass<C, 8, E>(p, act, g0, N, Ns, tw, warp); Ns *= 8; }
+  }
+#pragma unroll 1
+  for (int n = 0; n < L / LE; ++n) { stockham_pass<C, E, E>(p, act, g0, N, Ns, tw, warp); Ns *= E; }
+}
+
+struct FftPad16 { __device__ __forceinline__ int operator()(int e) const { return fft_pad<double2>(e); } };
+
+// Forward transforms, in place, of nlines lines of padded length NP that start `off` values behind
+// the start of the dynamic shared memory, which holds the twiddle table.  Every thread of the
+// block calls it, the lines complete in shared memory; they are complete again on return.
+//
+// A line belongs to N/E consecutive threads.  When these are within one warp (N/E <= 32: lines up
+// to 256 with 8 elements per thread) its passes need no block barrier, only the warp's; before,
+// each pass waited twice for the whole block (24-27% of the stalls of the 256^2 passes).
+//
+// An inverse transform is the forward one of values with real and imaginary part exchanged,
+// exchanged again (swp below), so that one inlined copy serves every transform of a kernel:
+// unrolled passes are 10 to 20 KB of instructions, run once or twice by a block, and a third of
+// the stalls of the FP64 column passes was waiting for them (ncu, no_instruction) with three.
+template <class C, int E>
+__device__ __forceinline__ void fft_lines_e(int off, int nlines, int NP, int L) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int s_key[32];
+  const C* tw = reinterpret_cast<const C*>(smem_raw);
+  C* buf = reinterpret_cast<C*>(smem_raw) + off;
+  const int LG = L - (E == 16 ? 4 : E == 8 ? 3 : E == 4 ? 2 : 1);   // log2 of the threads of a line
+  const int per = blockDim.x >> LG;
+  const int q0 = threadIdx.x >> LG, g0 = threadIdx.x & ((1 << LG) - 1);
+  const bool warp = LG <= 5;
+#pragma unroll 1
+  for (int b = 0; b < nlines; b += per) {
+    const int q = b + q0;
+    const bool act = q0 < per && q < nlines;
+    C* p = buf + (act ? q : 0) * NP;
+    int g = g0;
+    asm volatile("" : "+r"(g));   // keeps every pass's addresses from being computed ahead of the loop, into spills
+    if constexpr (sizeof(C) == 16)
+      fx_fft<E>(reinterpret_cast<FxC*>(p), act, g, L, reinterpret_cast<const FxW*>(tw), s_key, warp, FftPad16{});
+    else
+      stockham_fft<C, E>(p, act, g, L, tw, warp);
   }
   __syncthreads();
 }
 
-// Full transform of length N = 2^L (N >= E) for the NI lines of this thread, E
-// elements per thread and pass (E in {2, 4, 8, 16}: radix-E passes plus one smaller
-// pass when log2 N is not a multiple of log2 E).  Threads with g0 >= N/E (or
-// inactive items) only join the barriers.
-template <class C, bool INV, int E, int NI>
-__device__ __forceinline__ void stockham_fft(C* const (&lines)[NI], const bool (&active_in)[NI], int g0, int es, int L,
-                                             const C* tw) {
-  const int N = 1 << L;
-  bool active[NI];
-#pragma unroll
-  for (int it = 0; it < NI; ++it) active[it] = active_in[it] && g0 < (N / E);
-  int Ns = 1;
-  constexpr int LE = (E == 16) ? 4 : (E == 8) ? 3 : (E == 4) ? 2 : 1;
-  const int rem = L % LE;
-  if (rem == 1) { stockham_pass<C, INV, 2, E, NI>(lines, active, g0, es, N, Ns, tw); Ns *= 2; }
-  else if (rem == 2) { stockham_pass<C, INV, 4, E, NI>(lines, active, g0, es, N, Ns, tw); Ns *= 4; }
-  else if constexpr (E == 16) {
-    if (rem == 3) { stockham_pass<C, INV, 8, E, NI>(lines, active, g0, es, N, Ns, tw); Ns *= 8; }
-  }
-  for (int p = 0; p < L / LE; ++p) { stockham_pass<C, INV, E, E, NI>(lines, active, g0, es, N, Ns, tw); Ns *= E; }
+// real and imaginary part exchanged
+template <class C> __device__ __forceinline__ C swp(C a) {
+  C r;
+  r.x = a.y;
+  r.y = a.x;
+  return r;
 }
 
 }  // namespace gpsoc

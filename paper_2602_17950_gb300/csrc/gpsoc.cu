@@ -139,7 +139,6 @@ struct gpsoc_problem {
   size_t tmp_len = 0;
   Bufs<double> b64;
   Bufs<float> b32;              // FP32 working set of mixed-precision solves (allocated on first use)
-  std::map<int, double2*> tw64;
   std::map<int, float2*> tw32;
   int level = 0;
   bool has_state = false;
@@ -224,48 +223,29 @@ TrapDev make_trap(const gpsoc_problem* p, int level) {
   return t;
 }
 
-gpsoc_status twiddles(gpsoc_problem* p, int n, const double2** out) {
-  auto it = p->tw64.find(n);
-  if (it != p->tw64.end()) { *out = it->second; return GPSOC_OK; }
+// twiddle table of the FP32 passes (the FP64 ones have theirs in fixfft.cuh)
+gpsoc_status twiddles(gpsoc_problem* p, int n, const float2** out) {
+  auto it = p->tw32.find(n);
+  if (it != p->tw32.end()) { *out = it->second; return GPSOC_OK; }
   // W_n^k = exp(-2 pi i k / n), k < n; from the first octant by symmetry so that
   // W^(n/4) = -i, W^(n/2) = -1 hold exactly
-  std::vector<double2> h(n);
+  std::vector<float2> h(n);
   const double PI = 3.14159265358979323846;
   for (int k = 0; k < n; ++k) {
     int m = k;
-    double sc = 1.0, ss = 1.0;
     // reduce to [0, n/4]: W^(k) = -i W^(k - n/4)
     int quad = 0;
     while (m > n / 4) { m -= n / 4; ++quad; }
     double c, sn;
     if (2 * m <= n / 4) { const double a = 2.0 * PI * m / n; c = std::cos(a); sn = std::sin(a); }
     else { const double a = 2.0 * PI * (n / 4 - m) / n; c = std::sin(a); sn = std::cos(a); }
-    (void)sc; (void)ss;
     double re = c, im = -sn;   // exp(-i a)
     for (int q = 0; q < quad; ++q) { const double t = re; re = im; im = -t; }   // multiply by -i
-    h[k] = make_double2(re, im);
+    h[k] = make_float2((float)re, (float)im);
   }
-  double2* d = nullptr;
-  CK(cudaMalloc(&d, sizeof(double2) * n));
-  CK(cudaMemcpy(d, h.data(), sizeof(double2) * n, cudaMemcpyHostToDevice));
-  p->tw64[n] = d;
-  *out = d;
-  return GPSOC_OK;
-}
-
-gpsoc_status twiddles(gpsoc_problem* p, int n, const float2** out) {
-  auto it = p->tw32.find(n);
-  if (it != p->tw32.end()) { *out = it->second; return GPSOC_OK; }
-  const double2* d64;
-  gpsoc_status s = twiddles(p, n, &d64);
-  if (s != GPSOC_OK) return s;
-  std::vector<double2> h(n);
-  CK(cudaMemcpy(h.data(), d64, sizeof(double2) * n, cudaMemcpyDeviceToHost));
-  std::vector<float2> f(n);
-  for (int k = 0; k < n; ++k) f[k] = make_float2((float)h[k].x, (float)h[k].y);
   float2* d = nullptr;
   CK(cudaMalloc(&d, sizeof(float2) * n));
-  CK(cudaMemcpy(d, f.data(), sizeof(float2) * n, cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(d, h.data(), sizeof(float2) * n, cudaMemcpyHostToDevice));
   p->tw32[n] = d;
   *out = d;
   return GPSOC_OK;
@@ -288,12 +268,10 @@ gpsoc_status chain_args(gpsoc_problem* p, int level, ChainArgs<T>& a) {
   a.gate = GATE_ACTIVE;
   a.scale = 1.0;
   a.cnt = p->d_cnt;
-  for (int i = 0; i < 3; ++i) {
-    if (i < p->dim) {
-      const cx_t<T>* tw;
-      gpsoc_status s = twiddles(p, a.g.n[i], &tw);
+  if constexpr (sizeof(T) == 4) {
+    for (int i = 0; i < p->dim; ++i) {
+      gpsoc_status s = twiddles(p, a.g.n[i], &a.tw[i]);
       if (s != GPSOC_OK) return s;
-      a.tw[i] = tw;
     }
   }
   return GPSOC_OK;
@@ -1210,9 +1188,8 @@ gpsoc_status gpsoc_create(const gpsoc_grid* grid, const gpsoc_trap* trap, const 
   // twiddle tables of every axis length of every level (no allocation later, e.g. during graph capture)
   for (int lev = 0; lev <= p->max_level; ++lev) {
     for (int i = 0; i < p->dim; ++i) {
-      const double2* tw;
-      const float2* tw32;
-      if (twiddles(p, p->n[i] >> lev, &tw) != GPSOC_OK || twiddles(p, p->n[i] >> lev, &tw32) != GPSOC_OK)
+      const float2* tw;
+      if (twiddles(p, p->n[i] >> lev, &tw) != GPSOC_OK)
         return bail(GPSOC_ENOMEM, "twiddle setup failed");
     }
   }
@@ -1235,7 +1212,6 @@ void gpsoc_destroy(gpsoc_problem* p) {
   float2* arrs32[] = {p->b32.Phi, p->b32.HPhi, p->b32.R[0], p->b32.R[1], p->b32.P[0], p->b32.P[1],
                       p->b32.Z, p->b32.D, p->b32.A, p->b32.B, p->b32.W, p->b32.G, p->b32.Xh, p->b32.Ph};
   for (float2* a : arrs32) if (a) cudaFree(a);
-  for (auto& kv : p->tw64) cudaFree(kv.second);
   for (auto& kv : p->tw32) cudaFree(kv.second);
   if (p->d_part) cudaFree(p->d_part);
   if (p->d_st) cudaFree(p->d_st);

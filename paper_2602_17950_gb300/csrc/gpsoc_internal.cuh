@@ -181,7 +181,7 @@ struct ChainArgs {
   const C* in0; const C* in1; const C* in2; const C* in3; const C* in4;
   C* out0; C* out1;
   double* part; int pmax;
-  const C* tw[3];     // twiddle tables exp(-2 pi i k / n_axis), k < n_axis/2
+  const C* tw[3];     // FP32 passes: twiddle tables exp(-2 pi i k / n_axis), k < n_axis
   int gate;
   int nsolve;
   double scale;       // extra scale factor (prolongation, normalisation)

@@ -112,7 +112,7 @@ extern "C" gpsoc_status gpsoc_apply_h_noalloc(const gpsoc_grid* grid, const gpso
     g.log2n[i] = ilog2i(g.n[i]);
     g.npts *= g.n[i];
   }
-  // scratch layout: A, B, W, G arrays | partial sums | states | parameters | twiddles | observables
+  // scratch layout: A, B, W, G arrays | partial sums | states | parameters | observables
   const size_t arr = sizeof(double2) * (size_t)batch * 3 * g.npts;
   const int nb_row = row_blocks_per_solve<double>(g, batch);
   int pmax = nb_row;
@@ -122,8 +122,7 @@ extern "C" gpsoc_status gpsoc_apply_h_noalloc(const gpsoc_grid* grid, const gpso
   const size_t o_part = off; off += align256(sizeof(double) * (size_t)batch * NSLOT * pmax);
   const size_t o_st = off; off += align256(sizeof(SolveState) * batch);
   const size_t o_ph = off; off += align256(sizeof(PhysDev) * batch);
-  size_t o_tw[3];
-  for (int i = 0; i < g.d; ++i) { o_tw[i] = off; off += align256(sizeof(double2) * g.n[i]); }
+  for (int i = 0; i < g.d; ++i) off += align256(sizeof(double2) * g.n[i]);   // spare; part of the budget callers know
   const size_t o_obs = off; off += align256(sizeof(double) * 9 * batch);
   if (off > kNoAllocScratchBytes) {
     return GPSOC_EBUDGET;
@@ -140,7 +139,7 @@ extern "C" gpsoc_status gpsoc_apply_h_noalloc(const gpsoc_grid* grid, const gpso
   SolveState* sst = (SolveState*)(base + o_st);
   PhysDev* ph = (PhysDev*)(base + o_ph);
   double* dobs = (double*)(base + o_obs);
-  // parameters and twiddle tables from stack buffers (copied before cudaMemcpyAsync returns)
+  // parameters from a stack buffer (copied before cudaMemcpyAsync returns)
   PhysDev phs[64];
   for (int b0 = 0; b0 < batch; b0 += 64) {
     const int nb = std::min(64, batch - b0);
@@ -154,26 +153,7 @@ extern "C" gpsoc_status gpsoc_apply_h_noalloc(const gpsoc_grid* grid, const gpso
     e = cudaMemcpyAsync(ph + b0, phs, sizeof(PhysDev) * nb, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return GPSOC_ECUDA;
   }
-  double2 tw[1024];
-  const double PI = 3.14159265358979323846;
   ChainArgs<double> a{};
-  for (int i = 0; i < g.d; ++i) {
-    const int n = g.n[i];
-    for (int k = 0; k < n; ++k) {
-      // exp(-2 pi i k / n) from the first octant by symmetry (exact at multiples of n/4)
-      int m = k, quad = 0;
-      while (m > n / 4) { m -= n / 4; ++quad; }
-      double c, sn;
-      if (2 * m <= n / 4) { const double ang = 2.0 * PI * m / n; c = std::cos(ang); sn = std::sin(ang); }
-      else { const double ang = 2.0 * PI * (n / 4 - m) / n; c = std::sin(ang); sn = std::cos(ang); }
-      double re = c, im = -sn;
-      for (int q = 0; q < quad; ++q) { const double t = re; re = im; im = -t; }
-      tw[k] = make_double2(re, im);
-    }
-    e = cudaMemcpyAsync(base + o_tw[i], tw, sizeof(double2) * n, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return GPSOC_ECUDA;
-    a.tw[i] = (const double2*)(base + o_tw[i]);
-  }
   k_init_state<<<(batch + 127) / 128, 128, 0, st>>>(sst, batch);
   a.g = g;
   for (int i = 0; i < 3; ++i) a.trap.half_g2[i] = (i < g.d) ? 0.5 * trap->g[i] * trap->g[i] : 0.0;
