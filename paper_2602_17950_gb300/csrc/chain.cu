@@ -17,6 +17,7 @@
 // inverse (y is constant along an x row), the x D_y piece is carried as a
 // second array G = F_y^{-1}[v_y F_y A] and multiplied by x after the x inverse.
 #include <map>
+#include <type_traits>
 #include <mutex>
 
 #include "gpsoc_internal.cuh"
@@ -94,8 +95,10 @@ __device__ __forceinline__ void store_partials(const W (&acc)[K], const int (&sl
   double v[K];
   if constexpr (sizeof(W) == 4 && K >= 2) {
     block_reduce_df<K>(acc, v, red);     // FP32 partials: double-float sums on the FP32 pipes
-  } else if constexpr (sizeof(W) == 4) {
-    v[0] = block_reduce1_f(acc[0], mx[0], red);
+  } else if constexpr (K == 1 && sizeof(W) == 4) {
+    v[0] = mx[0] ? block_max((double)acc[0], red) : block_sum_f(acc[0], red);
+  } else if (K == 1 && mx[0]) {
+    v[0] = block_max(acc[0], red);
   } else {
 #pragma unroll
     for (int k = 0; k < K; ++k) v[k] = (double)acc[k];
@@ -130,6 +133,10 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
   constexpr bool two = (MODE == ROW_INV_H || MODE == ROW_INV_P || MODE == ROW_INV_LIN || MODE == ROW_INV_P_HY);
   C* buf1 = buf0 + 3 * CP;
   double* red = (double*)(buf1 + (two ? 3 * CP : 0));
+  // scratch of a fused scalar step: over the tile, which is done with by then (32 doubles per warp are
+  // at most half of its 24 or 48 bytes per element)
+  double* tail = (double*)smem_raw;
+  using PV = std::conditional_t<sizeof(T) == 4, DF, double>;   // format of the sum partials
   const long long sbase = (long long)s * 3 * npts;
   const long long rbase = (long long)rb * R * nx;   // offset of the tile inside a component
   const long long sslot = (long long)s * NSLOT;
@@ -207,7 +214,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
           const double rr = h.x - mu64 * f[c].x, ri = h.y - mu64 * f[c].y;
           const C rc = mk<C>(rr, ri);
           A.out1[sbase + c * npts + off] = rc;
-          acc[0] = fmax(acc[0], (W)sqrt((W)(rr * rr + ri * ri)));
+          acc[0] = fmax(acc[0], rc.x * rc.x + rc.y * rc.y);
           W den = al[c] + V + c0 * rhow;
           den = fmax(den, (W)1e-12 * al[c]);
           const W sc = use_pv ? rsqrt_w<W>(den) : (W)1;
@@ -232,7 +239,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
           rr.x = h[c].x - mu * f[c].x;
           rr.y = h[c].y - mu * f[c].y;
           A.out1[sbase + c * npts + off] = rr;
-          acc[0] = fmax(acc[0], sqrt(rr.x * rr.x + rr.y * rr.y));
+          acc[0] = fmax(acc[0], rr.x * rr.x + rr.y * rr.y);
           W den = al[c] + V + c0 * rho;
           den = fmax(den, (W)1e-12 * al[c]);
           const W sc = use_pv ? rsqrt_w<W>(den) : (W)1;
@@ -254,7 +261,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
       store_partials<1, W>(acc, slots, mx, red, A.part, sslot, A.pmax, rb);
     }
     if ((MODE == ROW_FWD_PRE || MODE == ROW_FWD_PRE_HY) && A.fuse && last_block(A.cnt, s, bps, &last_flag))
-      sc_res(A.sc, s, red);
+      sc_res(A.sc, s, tail);
     return;
   }
 
@@ -331,7 +338,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
     const bool mx[5] = {false, false, false, false, false};
     const int slots[5] = {SL_RZ, SL_RPZ, SL_ZPHI, SL_PPHI, SL_RP};
     store_partials<5, W>(acc, slots, mx, red, A.part, sslot, A.pmax, rb);
-    if (A.fuse && last_block(A.cnt, s, bps, &last_flag)) sc_beta(A.sc, s, red);
+    if (A.fuse && last_block(A.cnt, s, bps, &last_flag)) sc_beta<PV>(A.sc, s, tail);
     return;
   }
 
@@ -456,7 +463,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
     const bool mx12[12] = {};
     const int slots[12] = {SL_Q, SL_RHO2, SL_F2, SL_V0, SL_V1, SL_V2, SL_C0, SL_C1, SL_C2, SL_M0, SL_M1, SL_M2};
     store_partials<12, W>(a12, slots, mx12, red, A.part, sslot, A.pmax, rb);
-    if (A.fuse && last_block(A.cnt, s, bps, &last_flag)) sc_obs(A.sc, s, red);
+    if (A.fuse && last_block(A.cnt, s, bps, &last_flag)) sc_obs<PV>(A.sc, s, tail);
   } else {
     const int slots[13] = {SL_HPP, SL_HPHIP, SL_RPHI, SL_IFR, SL_IFP, SL_IRR, SL_IRP, SL_IPP,
                            SL_JFR, SL_JFP, SL_JRR, SL_JRP, SL_JPP};
@@ -470,7 +477,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
       __syncthreads();   // thread 0 of store_partials wrote SL_RPHI's FP32 sum before
       put_partials<2>(A.part, sslot, A.pmax, rb, slots2, v2, mx2, true);
     }
-    if (A.fuse && last_block(A.cnt, s, bps, &last_flag)) sc_step(A.sc, s, red);
+    if (A.fuse && last_block(A.cnt, s, bps, &last_flag)) sc_step<PV>(A.sc, s, tail);
   }
 }
 

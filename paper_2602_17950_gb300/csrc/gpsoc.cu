@@ -107,8 +107,7 @@ const char* col_name(int m, int axis) {
   return (m >= 0 && m < 7) ? n[axis == 2 ? 1 : 0][m] : "col_?";
 }
 const char* scalar_name(int ph) {
-  static const char* n[] = {"sc_init", "sc_obs", "sc_res", "sc_beta", "sc_step", "sc_clear",
-                            "sc_norm", "sc_model", "sc_kin"};
+  static const char* n[] = {"sc_init", "sc_obs", "sc_clear", "sc_norm", "sc_model", "sc_kin"};
   return (ph >= 0 && ph < (int)(sizeof(n) / sizeof(n[0]))) ? n[ph] : "sc_?";
 }
 const char* elem_name(int m) {

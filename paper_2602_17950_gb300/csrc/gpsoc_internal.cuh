@@ -98,8 +98,8 @@ struct SolveState {
   double res_inf, dphi_inf;
   // PCG scalars
   double s_prev, s_cur, beta, cproj;
-  double P2, HPP, HPhiP, RPhi;
-  double I[6], J[6];
+  double P2, HPP, HPhiP;
+  double K[6];              // c0 I + c1 J of the density and spin integrals of the step (energy_change_sc)
   double a, b, theta, dE, dE_last;
   double upd_c, upd_s, upd_scale;
   double E_win;     // FP32 phase: energy when the stall window opened
@@ -247,23 +247,20 @@ __device__ __forceinline__ bool gate_ok(const SolveState* st, int gate, int s) {
 }
 
 // True in every thread of the block that arrives last among the `bps` blocks of
-// solve s (threadfence-reduction pattern: partial sums written before the
-// arrival are visible to the last block).  The last block resets the counter.
+// solve s; the partial sums written before the arrival are visible to it, and it resets the counter.
+// One thread's acquire-release addition orders the whole block's writes before it (they precede the
+// barrier) and the block's reads after it.
 __device__ __forceinline__ bool last_block(unsigned* cnt, int s, int bps, int* flag_smem) {
   pdl_trigger();
-  __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
-    const unsigned prev = atomicAdd(cnt + s, 1u);
+    unsigned prev;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(prev) : "l"(cnt + s) : "memory");
     *flag_smem = (prev == (unsigned)bps - 1u);
+    if (prev == (unsigned)bps - 1u) cnt[s] = 0u;
   }
   __syncthreads();
-  const bool last = *flag_smem != 0;
-  if (last) {
-    __threadfence();
-    if (threadIdx.x == 0) cnt[s] = 0u;
-  }
-  return last;
+  return *flag_smem != 0;
 }
 
 // wavenumber v_p = pi p / L of FFT index k on an axis of n points (Section 3.2),
@@ -389,31 +386,37 @@ __device__ __forceinline__ DF df_shfl_xor(DF a, int ofs) {
   return r;
 }
 
-// One FP32 block total (a sum in double-float, or a max in FP32, which is exact),
-// rounded to FP64 once.  scratch: >= blockDim.x / 32 + 1 doubles.
-__device__ __forceinline__ double block_reduce1_f(float a, bool is_max, double* scratch) {
+// One FP32 block sum in double words, rounded to FP64 once.  scratch: >= blockDim.x / 32 doubles.
+__device__ __forceinline__ double block_sum_f(float a, double* scratch) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
   __syncthreads();  // scratch may alias shared memory the caller used just before
   DF x{a, 0.0f};
 #pragma unroll
-  for (int ofs = 16; ofs > 0; ofs >>= 1) {
-    const DF o = df_shfl_xor(x, ofs);
-    if (is_max) x.hi = fmaxf(x.hi, o.hi);
-    else x = df_add(x, o);
-  }
+  for (int ofs = 16; ofs > 0; ofs >>= 1) x = df_add(x, df_shfl_xor(x, ofs));
   float2* sc2 = reinterpret_cast<float2*>(scratch);
-  if (lane == 0) sc2[warp] = make_float2(x.hi, is_max ? 0.0f : x.lo);
+  if (lane == 0) sc2[warp] = make_float2(x.hi, x.lo);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    DF acc{sc2[0].x, sc2[0].y};
-    for (int w = 1; w < nw; ++w) {
-      if (is_max) acc.hi = fmaxf(acc.hi, sc2[w].x);
-      else acc = df_add(acc, DF{sc2[w].x, sc2[w].y});
-    }
-    scratch[nw] = (double)acc.hi + (double)acc.lo;
-  }
+  DF acc{sc2[0].x, sc2[0].y};
+  for (int w = 1; w < nw; ++w) acc = df_add(acc, DF{sc2[w].x, sc2[w].y});
+  return (double)acc.hi + (double)acc.lo;
+}
+
+// warp and block maximum of values that are not negative, which are ordered as their bits (an FP64
+// comparison holds the FP64 pipe for 64 cycles).  scratch: >= blockDim.x / 32 doubles.
+__device__ __forceinline__ unsigned long long warp_max(unsigned long long m) {
+  const unsigned h = __reduce_max_sync(0xffffffffu, (unsigned)(m >> 32));
+  const unsigned l = __reduce_max_sync(0xffffffffu, (unsigned)(m >> 32) == h ? (unsigned)m : 0u);
+  return ((unsigned long long)h << 32) | l;
+}
+__device__ __forceinline__ double block_max(double x, double* scratch) {
+  __syncthreads();  // scratch may alias shared memory the caller used just before
+  const unsigned long long m = warp_max((unsigned long long)__double_as_longlong(x));
+  auto* sc = reinterpret_cast<unsigned long long*>(scratch);
+  if ((threadIdx.x & 31) == 0) sc[threadIdx.x >> 5] = m;
   __syncthreads();
-  return scratch[nw];
+  unsigned long long r = sc[0];
+  for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r = sc[w] > r ? sc[w] : r;
+  return __longlong_as_double((long long)r);
 }
 
 // Block sums of double-float per-thread partials, same fixed order and same

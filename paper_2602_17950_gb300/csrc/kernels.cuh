@@ -8,9 +8,6 @@ namespace gpsoc {
 enum Phase {
   PH_INIT = 0,      // reset per-level flags (flags & 1: also reset counters)
   PH_OBS,           // E, mu, alpha, masses from the H-chain partials
-  PH_RES,           // max |r| and the stopping test
-  PH_BETA,          // Polak-Ribiere+ beta, Re<D, Phi> and the beta = 0 decision of Algorithm 2 Step 2
-  PH_STEP,          // Algorithm 2 (step model, backtracking, update coefficients)
   PH_CLEAR,         // drop the pending-step flag
   PH_NORM,          // 1/sqrt(mass) per solve into norm_scale
   PH_MODEL,         // a_n, b_n and E(theta) - E(0) at given angles into model_out
@@ -25,7 +22,7 @@ struct ScalarArgs {
   int nb_row, nb_col;
   int nsolve;
   int phase;
-  int flags;          // PH_INIT: 1 = reset counters, 4 = keep the direction; PH_STEP: 2 = count as an FP32 iteration
+  int flags;          // PH_INIT: 1 = reset counters, 4 = keep the direction; PH_OBS: as ScalarCtx
   long long npts;
   double dV;
   OptsDev opts;

@@ -20,7 +20,7 @@ namespace gpsoc {
 static constexpr int kScalarThreads = 128;
 
 __global__ void k_scalar(ScalarArgs A) {
-  __shared__ double scratch[16 * 8 + 16];
+  __shared__ double scratch[32 * (kScalarThreads / 32) + 1];
   pdl_wait();
   const int s = blockIdx.x;
   if (s >= A.nsolve) return;
@@ -42,36 +42,34 @@ __global__ void k_scalar(ScalarArgs A) {
       }
       return;
     case PH_NORM: {
-      double v[1];
       const int sl[1] = {SL_NORM};
-      slot_totals<1>(X, s, sl, A.nb_row, v, scratch);
-      if (threadIdx.x == 0) A.norm_scale[s] = (v[0] > 0.0 && isfinite(v[0])) ? 1.0 / sqrt(v[0] * A.dV) : 0.0;
+      slot_totals<double, 1, 1>(X, s, sl, A.nb_row, 0, -1, scratch);
+      const double v = scratch[0];
+      if (threadIdx.x == 0) A.norm_scale[s] = (v > 0.0 && isfinite(v)) ? 1.0 / sqrt(v * A.dV) : 0.0;
       return;
     }
-    case PH_OBS: sc_obs(X, s, scratch); return;
-    case PH_RES: sc_res(X, s, scratch); return;
-    case PH_BETA: sc_beta(X, s, scratch); return;
-    case PH_STEP: sc_step(X, s, scratch); return;
+    case PH_OBS:
+      if (A.part_dw) sc_obs<DF>(X, s, scratch); else sc_obs<double>(X, s, scratch);
+      return;
     case PH_CLEAR: if (threadIdx.x == 0) S.pending = 0; return;
     case PH_KIN: {
-      double kin[3];
       const int ks[3] = {SL_KIN0, SL_KIN1, SL_KIN2};
-      slot_totals<3>(X, s, ks, A.nb_col, kin, scratch);
-      if (threadIdx.x == 0) for (int c = 0; c < 3; ++c) S.kin[c] = kin[c];
+      slot_totals<double, 3, 3>(X, s, ks, A.nb_col, 0, -1, scratch);
+      if (threadIdx.x < 3) S.kin[threadIdx.x] = scratch[threadIdx.x];
       return;
     }
     case PH_MODEL: {
-      SolveState L;
-      if (threadIdx.x == 0) L = S;
-      PNorm pn;
-      step_sums(X, s, scratch, L, pn);
-      if (threadIdx.x == 0) {
-        S = L;
-        const PhysDev ph = A.phys[s];
-        double* o = A.model_out + (long long)s * (2 + A.n_theta);
-        o[0] = L.a; o[1] = L.b;
-        for (int k = 0; k < A.n_theta; ++k) o[2 + k] = energy_change(L, ph.c0, ph.c1, A.thetas[k]);
-      }
+      __shared__ SolveState L;
+      state_load(L, &S);
+      const int sl[kStepSlots] = {GPSOC_STEP_SLOTS};
+      if (A.part_dw) slot_totals<DF, kStepSlots, kStepSlots>(X, s, sl, A.nb_row, 0, -1, scratch);
+      else slot_totals<double, kStepSlots, kStepSlots>(X, s, sl, A.nb_row, 0, -1, scratch);
+      if (threadIdx.x >= 32) return;
+      step_sums(X, s, scratch, L);
+      state_store_warp(&S, L);
+      double* o = A.model_out + (long long)s * (2 + A.n_theta);
+      if (threadIdx.x == 0) { o[0] = L.a; o[1] = L.b; }
+      for (int k = threadIdx.x; k < A.n_theta; k += 32) o[2 + k] = energy_change(L, A.thetas[k]);
       return;
     }
   }
@@ -263,7 +261,7 @@ __global__ void __launch_bounds__(kHyThreads, kHyBlocksPerSM) k_hy_upd(HyArgs A)
   }
   double* P = A.part + (long long)s * NSLOT * A.pmax + rb;
   if (upd) {
-    const double v = block_reduce1_f(dmax, true, scratch);
+    const double v = block_max((double)dmax, scratch);
     if (threadIdx.x == 0) put_partial(P + (long long)SL_DPHIINF * A.pmax, v, true, true);
   }
   if (!red) return;
