@@ -83,9 +83,23 @@ __device__ __forceinline__ void spin_a(C1 p1, C2 p0, C3 pm, W& ar, W& ai) {
   ai = (W)p0.x * (W)p1.y - (W)p0.y * (W)p1.x + (W)pm.x * (W)p0.y - (W)pm.y * (W)p0.x;
 }
 
-template <class W> __device__ __forceinline__ W rsqrt_w(W x);
-template <> __device__ __forceinline__ double rsqrt_w<double>(double x) { return rsqrt(x); }
-template <> __device__ __forceinline__ float rsqrt_w<float>(float x) { return rsqrtf(x); }
+// 1/sqrt(x), x > 0.  FP64: the FP32 value as a start (the integer pipes convert), then
+// y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2, |e| < 2^-20, to e^3: 5 FP64 instructions against 9 of the
+// library's; outside the FP32 range the library
+__device__ __forceinline__ float rsqrt_w(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double rsqrt_w(double x) {
+  const int h = __double2hiint(x);
+  if (h < 0x39000000 || h > 0x46f00000) return rsqrt(x);   // below 2^-111, above 2^112, or negative
+  const double y = widen_f(rsqrtf(narrow_f(x)));
+  const double e = 1.0 - (x * y) * y;
+  return y + y * (e * (0.375 * e + 0.5));
+}
+// larger of two values, the second positive: their bits are ordered alike (and a negative or
+// smaller first one is below), without the FP64 pipe
+__device__ __forceinline__ float max_pos(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double max_pos(double a, double b) {
+  return __double_as_longlong(a) < __double_as_longlong(b) ? b : a;
+}
 
 // write per-thread partial sums (working precision) as a deterministic block total in FP64
 // (FP32 partials are added in double-float, which carries more bits than the partials hold)
@@ -110,139 +124,167 @@ __device__ __forceinline__ void store_partials(const W (&acc)[K], const int (&sl
 // ============================================================== row passes (x axis)
 // Working precision W = T: FP64 kernels compute in double, FP32 kernels in float
 // (per-thread partial sums in T, block and grid reductions in FP64).
+//
+// Sizes are powers of two, so indices are split by shifts (integer divisions, two of them of 64 bits
+// per point, were a third of the instructions of the FP32 passes).  The tiles of the inverse passes
+// come by asynchronous copies, which are under way while the twiddle table is set up.
 template <class T, int MODE>
 __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) {
   using C = cx_t<T>;
   using W = T;
+  using PV = std::conditional_t<sizeof(T) == 4, DF, double>;   // format of the sum partials
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int last_flag;
-  const int nx = A.g.n[0], Lx = A.g.log2n[0];
+  constexpr bool fwd = (MODE == ROW_FWD_PLAIN || MODE == ROW_FWD_UPD || MODE == ROW_FWD_PROJ || MODE == ROW_FWD_PRE ||
+                        MODE == ROW_FWD_PRE_HY);
+  constexpr bool two = (MODE == ROW_INV_H || MODE == ROW_INV_P || MODE == ROW_INV_LIN || MODE == ROW_INV_P_HY);
+  const int nx = A.g.n[0], Lx = A.g.log2n[0], Ly = A.g.log2n[1], ny = A.g.n[1];
   const long long npts = A.g.npts;
-  const int rows = (int)(npts / nx);
-  const int bps = rows / R;
+  const int bps = (int)(npts >> Lx) / R;
   const int s = blockIdx.x / bps;
-  const int rb = blockIdx.x % bps;
-  C* s_tw = (C*)smem_raw;
-  load_tw<T>(s_tw, A.tw[0], nx, ept);   // constant table: before the wait on the previous kernel
+  const int rb = blockIdx.x - s * bps;
   pdl_wait();
   if (s >= A.nsolve || !gate_ok(A.st, A.gate, s)) return;
+  C* s_tw = (C*)smem_raw;
   const int b0 = fft_padded_len<C>(nx);   // the lines lie behind the table
   C* buf0 = s_tw + b0;
-  const int per = R * nx;             // elements of one component in the tile
-  const int NP = fft_padded_len<C>(nx), CP = R * NP;   // padded line length, component stride in smem
-  constexpr bool two = (MODE == ROW_INV_H || MODE == ROW_INV_P || MODE == ROW_INV_LIN || MODE == ROW_INV_P_HY);
+  const int per = R << Lx;            // elements of one component in the tile
+  const int NP = b0, CP = R * NP;     // padded line length, component stride in smem
   C* buf1 = buf0 + 3 * CP;
   double* red = (double*)(buf1 + (two ? 3 * CP : 0));
   // scratch of a fused scalar step: over the tile, which is done with by then (32 doubles per warp are
   // at most half of its 24 or 48 bytes per element)
   double* tail = (double*)smem_raw;
-  using PV = std::conditional_t<sizeof(T) == 4, DF, double>;   // format of the sum partials
-  const long long sbase = (long long)s * 3 * npts;
-  const long long rbase = (long long)rb * R * nx;   // offset of the tile inside a component
+  // this tile's first point; component c is npts further on
+  const long long base = (long long)s * 3 * npts + ((long long)rb * R << Lx);
+  const int row0 = rb * R;
   const long long sslot = (long long)s * NSLOT;
   const SolveState& S = A.st[s];
-  const PhysDev ph = A.phys[s];
-  const int ny = A.g.n[1];
+  const PhysDev& ph = A.phys[s];
 
-  if (MODE == ROW_FWD_PLAIN || MODE == ROW_FWD_UPD || MODE == ROW_FWD_PROJ || MODE == ROW_FWD_PRE ||
-      MODE == ROW_FWD_PRE_HY) {
+  if (!fwd || MODE == ROW_FWD_PLAIN) {
+    for (int e = threadIdx.x; e < per; e += blockDim.x) {
+      const int pos = (e >> Lx) * NP + fft_pad<C>(e & (nx - 1));
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        copy_async(&buf0[c * CP + pos], A.in0 + base + c * npts + e);
+        if (two) copy_async(&buf1[c * CP + pos], A.in1 + base + c * npts + e);
+      }
+    }
+  }
+  load_tw<T>(s_tw, A.tw[0], nx, ept);
+  // the solve's scalars, read before the transforms
+  const W c0 = pick<W>(ph.c0, ph.fc0), c1 = pick<W>(ph.c1, ph.fc1), Om = pick<W>(ph.Omega, ph.fOmega);
+  const W al[3] = {pick<W>(S.alpha[0], S.falpha[0]), pick<W>(S.alpha[1], S.falpha[1]), pick<W>(S.alpha[2], S.falpha[2])};
+  const int pk = A.sc.opts.precond;
+  const bool use_pv = (pk == GPSOC_PRECOND_COMBINED || pk == GPSOC_PRECOND_POTENTIAL);
+
+  if (fwd) {
     W acc[1] = {(W)0};
     const W cproj = pick<W>(S.cproj, S.fcproj), mu = A.given_r ? (W)0 : pick<W>(S.mu, S.fmu), beta = pick<W>(S.beta, S.fbeta);
-    const bool use_prev = (MODE == ROW_FWD_PROJ) && pick<W>(S.beta, S.fbeta) != (W)0;
+    const bool use_prev = (MODE == ROW_FWD_PROJ) && beta != (W)0;
     const bool upd = (MODE == ROW_FWD_UPD) && S.pending != 0;
-    const W uc = pick<W>(S.upd_c, S.fupd_c), us = pick<W>(S.upd_s, S.fupd_s), usc = pick<W>(S.upd_scale, S.fupd_scale);
-    const W al[3] = {pick<W>(S.alpha[0], S.falpha[0]), pick<W>(S.alpha[1], S.falpha[1]), pick<W>(S.alpha[2], S.falpha[2])};
-    const W c0 = pick<W>(ph.c0, ph.fc0);
-    for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int r = e / nx, j = e - r * nx;
-      const long long off = rbase + e;
+    const bool dphi = upd && A.sc.opts.stop == GPSOC_STOP_DPHI;   // only the stop1 test reads max |dPhi|
+    const W usc = pick<W>(S.upd_scale, S.fupd_scale);
+    const W uc = usc * pick<W>(S.upd_c, S.fupd_c), us = usc * pick<W>(S.upd_s, S.fupd_s);
+    const double mu64 = S.mu;
+    if (MODE == ROW_FWD_PLAIN) copy_wait();
+    else for (int e = threadIdx.x; e < per; e += blockDim.x) {
+      const int r = e >> Lx, j = e & (nx - 1);
+      const long long at = base + e;
       const int pos = r * NP + fft_pad<C>(j);
-      if (MODE == ROW_FWD_PLAIN) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) buf0[c * CP + pos] = A.in0[sbase + c * npts + off];
-      } else if (MODE == ROW_FWD_UPD) {
+      if (MODE == ROW_FWD_UPD) {
         // the step accepted by the previous iteration: Phi <- (cos t Phi + sin t P/|P|)/norm
-        // (Eqs. formula-pcg, update); reduce max |dPhi|^2 for the stop1 test
+        // (Eqs. formula-pcg, update); max |dPhi|^2 for the stop1 test
+        C f[3], p[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          C f = A.in0[sbase + c * npts + off];
+          f[c] = A.in0[at + c * npts];
+          if (upd) p[c] = __ldg(A.in2 + at + c * npts);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          C o = f[c];
           if (upd) {
-            const C p = A.in2[sbase + c * npts + off];
-            const C o = mk<C>(usc * (uc * f.x + us * p.x), usc * (uc * f.y + us * p.y));
-            const W dr = o.x - f.x, di = o.y - f.y;
-            acc[0] = fmax(acc[0], dr * dr + di * di);
-            A.out1[sbase + c * npts + off] = o;
-            f = o;
+            o = mk<C>(uc * f[c].x + us * p[c].x, uc * f[c].y + us * p[c].y);
+            if (dphi) {
+              const W dr = o.x - f[c].x, di = o.y - f[c].y;
+              acc[0] = max_pos(acc[0], dr * dr + di * di);
+            }
+            A.out1[at + c * npts] = o;
           }
-          buf0[c * CP + pos] = f;
+          buf0[c * CP + pos] = o;
         }
       } else if (MODE == ROW_FWD_PROJ) {
         // D = -z + beta P_prev, P = D - Re<D, Phi> Phi (Eq. formula-project); reduce ||P||^2
+        C z[3], f[3], q[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          const C z = A.in0[sbase + c * npts + off];
-          const C f = A.in1[sbase + c * npts + off];
-          W dr = -z.x, di = -z.y;
-          if (use_prev) { const C q = A.in2[sbase + c * npts + off]; dr += beta * q.x; di += beta * q.y; }
+          z[c] = __ldg(A.in0 + at + c * npts);
+          f[c] = __ldg(A.in1 + at + c * npts);
+          q[c] = use_prev ? __ldg(A.in2 + at + c * npts) : mk<C>((W)0, (W)0);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          W dr = -z[c].x, di = -z[c].y;
+          if (use_prev) { dr += beta * q[c].x; di += beta * q[c].y; }
           C p;
-          p.x = dr - cproj * f.x;
-          p.y = di - cproj * f.y;
-          A.out1[sbase + c * npts + off] = p;
+          p.x = dr - cproj * f[c].x;
+          p.y = di - cproj * f[c].y;
+          A.out1[at + c * npts] = p;
           acc[0] += p.x * p.x + p.y * p.y;
           buf0[c * CP + pos] = p;
         }
       } else if (MODE == ROW_FWD_PRE_HY) {
         // GPSOC_HYBRID: r = H Phi - mu Phi in FP64 from the FP64 state and H(Phi) (the residual
-        // keeps FP64 accuracy), stored as FP32; the preconditioner's transforms then run on
-        // P_V^{1/2} r in FP32
-        const int pk = A.sc.opts.precond;
-        const bool use_pv = (pk == GPSOC_PRECOND_COMBINED || pk == GPSOC_PRECOND_POTENTIAL);
-        const double mu64 = S.mu;
-        double2 f[3];
-        double rho = 0.0;
+        // keeps FP64 accuracy: one fused multiply-add each), stored as FP32; the preconditioner's
+        // transforms then run on P_V^{1/2} r in FP32, P_V from FP32 values as in the pass that
+        // closes them.  6 FP64 instructions a point (22 with rho and the conversions on that pipe,
+        // which bound the pass: 308k of its 397k cycles at 64 x 256^2)
+        double2 f[3], h[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          f[c] = A.phi64[sbase + c * npts + off];
-          rho += f[c].x * f[c].x + f[c].y * f[c].y;
+          f[c] = __ldg(A.phi64 + at + c * npts);
+          h[c] = __ldg(A.hl64 + at + c * npts);
         }
-        const long long row = off / nx;
-        const W V = trap_value<W>(A.trap, A.g, j, (int)(row % ny), (int)(row / ny), off);
-        const W rhow = (W)rho;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const double2 h = A.hl64[sbase + c * npts + off];
-          const double rr = h.x - mu64 * f[c].x, ri = h.y - mu64 * f[c].y;
-          const C rc = mk<C>(rr, ri);
-          A.out1[sbase + c * npts + off] = rc;
-          acc[0] = fmax(acc[0], rc.x * rc.x + rc.y * rc.y);
-          W den = al[c] + V + c0 * rhow;
-          den = fmax(den, (W)1e-12 * al[c]);
-          const W sc = use_pv ? rsqrt_w<W>(den) : (W)1;
-          buf0[c * CP + pos] = mk<C>(rc.x * sc, rc.y * sc);
-        }
-      } else {  // ROW_FWD_PRE: r = H Phi - mu Phi, then P_V^{1/2} r (Eq. PreCondPot)
-        const int pk = A.sc.opts.precond;
-        const bool use_pv = (pk == GPSOC_PRECOND_COMBINED || pk == GPSOC_PRECOND_POTENTIAL);
-        C f[3], h[3];
         W rho = (W)0;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          f[c] = A.in1[sbase + c * npts + off];
-          h[c] = A.in0[sbase + c * npts + off];
-          rho += f[c].x * f[c].x + f[c].y * f[c].y;
+          const W fx = narrow_f(f[c].x), fy = narrow_f(f[c].y);
+          rho += fx * fx + fy * fy;
         }
-        const long long row = off / nx;
-        const W V = trap_value<W>(A.trap, A.g, j, (int)(row % ny), (int)(row / ny), off);
+        const int row = row0 + r;
+        const W V = trap_value<W>(A.trap, A.g, j, row & (ny - 1), row >> Ly, at - (long long)s * 3 * npts);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const C rc = mk<C>(narrow_f(h[c].x - mu64 * f[c].x), narrow_f(h[c].y - mu64 * f[c].y));
+          A.out1[at + c * npts] = rc;
+          acc[0] = max_pos(acc[0], rc.x * rc.x + rc.y * rc.y);
+          const W den = max_pos(al[c] + (V + c0 * rho), (W)1e-12 * al[c]);
+          const W sc = use_pv ? rsqrt_w(den) : (W)1;
+          buf0[c * CP + pos] = mk<C>(rc.x * sc, rc.y * sc);
+        }
+      } else {  // ROW_FWD_PRE: r = H Phi - mu Phi, then P_V^{1/2} r (Eq. PreCondPot)
+        C f[3], h[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          f[c] = __ldg(A.in1 + at + c * npts);
+          h[c] = __ldg(A.in0 + at + c * npts);
+        }
+        W rho = (W)0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) rho += f[c].x * f[c].x + f[c].y * f[c].y;
+        const int row = row0 + r;
+        const W V = trap_value<W>(A.trap, A.g, j, row & (ny - 1), row >> Ly, at - (long long)s * 3 * npts);
+        const W w = V + c0 * rho;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           C rr;
           rr.x = h[c].x - mu * f[c].x;
           rr.y = h[c].y - mu * f[c].y;
-          A.out1[sbase + c * npts + off] = rr;
-          acc[0] = fmax(acc[0], rr.x * rr.x + rr.y * rr.y);
-          W den = al[c] + V + c0 * rho;
-          den = fmax(den, (W)1e-12 * al[c]);
-          const W sc = use_pv ? rsqrt_w<W>(den) : (W)1;
+          A.out1[at + c * npts] = rr;
+          acc[0] = max_pos(acc[0], rr.x * rr.x + rr.y * rr.y);
+          const W sc = use_pv ? rsqrt_w(max_pos(al[c] + w, (W)1e-12 * al[c])) : (W)1;
           buf0[c * CP + pos] = mk<C>(rr.x * sc, rr.y * sc);
         }
       }
@@ -250,11 +292,14 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
     __syncthreads();
     fft_lines<C>(b0, 3 * R, NP, Lx, ept);
     for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int pos = (e / nx) * NP + fft_pad<C>(e % nx);
+      const int pos = (e >> Lx) * NP + fft_pad<C>(e & (nx - 1));
 #pragma unroll
-      for (int c = 0; c < 3; ++c) A.out0[sbase + c * npts + rbase + e] = buf0[c * CP + pos];
+      for (int c = 0; c < 3; ++c) A.out0[base + c * npts + e] = buf0[c * CP + pos];
     }
-    if (MODE == ROW_FWD_PROJ || MODE == ROW_FWD_PRE || MODE == ROW_FWD_PRE_HY || (MODE == ROW_FWD_UPD && upd)) {
+    // GPSOC_HYBRID sums ||P||^2 with the step model, in more precision
+    const bool sum = (MODE == ROW_FWD_PROJ && !(A.sc.flags & 8)) || MODE == ROW_FWD_PRE || MODE == ROW_FWD_PRE_HY ||
+                     (MODE == ROW_FWD_UPD && dphi);
+    if (sum) {
       const bool mx[1] = {MODE != ROW_FWD_PROJ};
       const int slots[1] = {(MODE == ROW_FWD_PROJ) ? (int)SL_P2
                             : (MODE == ROW_FWD_PRE || MODE == ROW_FWD_PRE_HY) ? (int)SL_RINF : (int)SL_DPHIINF};
@@ -266,29 +311,20 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
   }
 
   // ---------------------------------------------------------------- inverse passes
-  // natural order in shared memory, inverse transform in place (both arrays' lines in one call)
-  for (int e = threadIdx.x; e < per; e += blockDim.x) {
-    const int pos = (e / nx) * NP + fft_pad<C>(e % nx);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      buf0[c * CP + pos] = swp(A.in0[sbase + c * npts + rbase + e]);
-      if (two) buf1[c * CP + pos] = swp(A.in1[sbase + c * npts + rbase + e]);
-    }
-  }
+  // forward transforms of both arrays' lines; the inverse ones are their values at index -j
+  copy_wait();
   __syncthreads();
   fft_lines<C>(b0, two ? 6 * R : 3 * R, NP, Lx, ept);
 
   const W inv_n = (W)1 / (W)npts;
-  const W Om = pick<W>(ph.Omega, ph.fOmega);
   if (MODE == ROW_INV_PLAIN) {
     const W sc = (W)A.scale;
     for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int r = e / nx, j = e - r * nx;
-      const int pos = r * NP + fft_pad<C>(j);
+      const int pos = (e >> Lx) * NP + fft_pad<C>(-e & (nx - 1));
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const C v = swp(buf0[c * CP + pos]);
-        A.out0[sbase + c * npts + rbase + e] = mk<C>(v.x * sc, v.y * sc);
+        const C v = buf0[c * CP + pos];
+        A.out0[base + c * npts + e] = mk<C>(v.x * sc, v.y * sc);
       }
     }
     return;
@@ -298,40 +334,38 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
     // Re<z, Phi>, Re<P_prev, Phi>, Re<r, P_prev> (the direction's projection and slope)
     W acc[5] = {(W)0, (W)0, (W)0, (W)0, (W)0};
     const bool use_prev = (A.in3 != nullptr) && !S.first;
-    const int pk = A.sc.opts.precond;
-    const bool use_pv = (pk == GPSOC_PRECOND_COMBINED || pk == GPSOC_PRECOND_POTENTIAL);
-    const W al[3] = {pick<W>(S.alpha[0], S.falpha[0]), pick<W>(S.alpha[1], S.falpha[1]), pick<W>(S.alpha[2], S.falpha[2])};
-    const W c0 = pick<W>(ph.c0, ph.fc0);
     for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int r = e / nx, j = e - r * nx;
-      const int pos = r * NP + fft_pad<C>(j);
-      const long long off = rbase + e;
+      const int r = e >> Lx, j = e & (nx - 1);
+      const int pos = r * NP + fft_pad<C>(-j & (nx - 1));
+      const long long at = base + e;
       W rho = (W)0;
-      C f[3];
+      C f[3], rr[3], rp[3], pp[3];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        f[c] = A.in1[sbase + c * npts + off];
-        rho += f[c].x * f[c].x + f[c].y * f[c].y;
+        f[c] = __ldg(A.in1 + at + c * npts);
+        rr[c] = __ldg(A.in2 + at + c * npts);
+        if (use_prev) {
+          rp[c] = __ldg(A.in3 + at + c * npts);
+          pp[c] = __ldg(A.in4 + at + c * npts);
+        }
       }
-      const long long row = off / nx;
-      const W V = trap_value<W>(A.trap, A.g, j, (int)(row % ny), (int)(row / ny), off);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) rho += f[c].x * f[c].x + f[c].y * f[c].y;
+      const int row = row0 + r;
+      const W V = trap_value<W>(A.trap, A.g, j, row & (ny - 1), row >> Ly, at - (long long)s * 3 * npts);
+      const W w = V + c0 * rho;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        W den = al[c] + V + c0 * rho;
-        den = fmax(den, (W)1e-12 * al[c]);
-        const W sc = use_pv ? inv_n * rsqrt_w<W>(den) : inv_n;
-        const C v = swp(buf0[c * CP + pos]);
+        const W sc = use_pv ? inv_n * rsqrt_w(max_pos(al[c] + w, (W)1e-12 * al[c])) : inv_n;
+        const C v = buf0[c * CP + pos];
         const C z = mk<C>(v.x * sc, v.y * sc);
-        A.out0[sbase + c * npts + off] = z;
-        const C rr = A.in2[sbase + c * npts + off];
-        acc[0] += rr.x * z.x + rr.y * z.y;
+        A.out0[at + c * npts] = z;
+        acc[0] += rr[c].x * z.x + rr[c].y * z.y;
         acc[2] += z.x * f[c].x + z.y * f[c].y;
         if (use_prev) {
-          const C rp = A.in3[sbase + c * npts + off];
-          const C pp = A.in4[sbase + c * npts + off];
-          acc[1] += rp.x * z.x + rp.y * z.y;
-          acc[3] += pp.x * f[c].x + pp.y * f[c].y;
-          acc[4] += rr.x * pp.x + rr.y * pp.y;
+          acc[1] += rp[c].x * z.x + rp[c].y * z.y;
+          acc[3] += pp[c].x * f[c].x + pp[c].y * f[c].y;
+          acc[4] += rr[c].x * pp[c].x + rr[c].y * pp[c].y;
         }
       }
     }
@@ -343,32 +377,42 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
   }
 
   // ROW_INV_H / ROW_INV_P / ROW_INV_LIN: lin = F_x^-1(T')/npts - Omega x F_x^-1(G)/npts + V u
-  const W c0 = pick<W>(ph.c0, ph.fc0), c1 = pick<W>(ph.c1, ph.fc1);
-  double rphi = 0.0, pp64 = 0.0;   // ROW_INV_P_HY: Re<P, Phi> against the FP64 Phi and ||P||^2, summed in FP64
-  W acc[13];
+  const W Omn = Om * inv_n;
+  DF rphi{0.0f, 0.0f}, pp{0.0f, 0.0f};   // ROW_INV_P_HY: Re<P, Phi> against the FP64 Phi and ||P||^2 in double words
+  W acc[12];
 #pragma unroll
-  for (int k = 0; k < 13; ++k) acc[k] = (W)0;
+  for (int k = 0; k < 12; ++k) acc[k] = (W)0;
+  W accR = (W)0;                         // ROW_INV_P: Re<P, Phi>
   for (int e = threadIdx.x; e < per; e += blockDim.x) {
-    const int r = e / nx, j = e - r * nx;
-    const int pos = r * NP + fft_pad<C>(j);
-    const long long off = rbase + e;
-    const long long row = off / nx;
-    const int iy = (int)(row % ny), iz = (int)(row / ny);
-    const W x = coord<W>(A.g, 0, j);
-    const W V = trap_value<W>(A.trap, A.g, j, iy, iz, off);
+    const int r = e >> Lx, j = e & (nx - 1);
+    const int pos = r * NP + fft_pad<C>(-j & (nx - 1));
+    const long long at = base + e;
+    const int row = row0 + r;
     C u[3];  // Phi for ROW_INV_H, P for ROW_INV_P / ROW_INV_LIN
+    C f[3], h[3];
+    double2 g64[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      u[c] = __ldg(A.in2 + at + c * npts);
+      if (MODE == ROW_INV_P || MODE == ROW_INV_P_HY) {
+        f[c] = __ldg(A.in3 + at + c * npts);
+        h[c] = __ldg(A.in4 + at + c * npts);
+      }
+      if (MODE == ROW_INV_P_HY) g64[c] = __ldg(A.phi64 + at + c * npts);
+    }
+    const W ox = Omn * coord<W>(A.g, 0, j);
+    const W V = trap_value<W>(A.trap, A.g, j, row & (ny - 1), row >> Ly, at - (long long)s * 3 * npts);
     W lin_r[3], lin_i[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      u[c] = A.in2[sbase + c * npts + off];
-      const C t = swp(buf0[c * CP + pos]);
-      const C gg = swp(buf1[c * CP + pos]);
-      lin_r[c] = (t.x - Om * x * gg.x) * inv_n + V * u[c].x;
-      lin_i[c] = (t.y - Om * x * gg.y) * inv_n + V * u[c].y;
+      const C t = buf0[c * CP + pos];
+      const C gg = buf1[c * CP + pos];
+      lin_r[c] = (t.x * inv_n - ox * gg.x) + V * u[c].x;
+      lin_i[c] = (t.y * inv_n - ox * gg.y) + V * u[c].y;
     }
     if (MODE == ROW_INV_LIN) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) A.out0[sbase + c * npts + off] = mk<C>(lin_r[c], lin_i[c]);
+      for (int c = 0; c < 3; ++c) A.out0[at + c * npts] = mk<C>(lin_r[c], lin_i[c]);
       continue;
     }
     if (MODE == ROW_INV_H) {
@@ -380,42 +424,37 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
       W ax, ay;
       spin_a<W>(u[0], u[1], u[2], ax, ay);
       const W Fz = m[0] - m[2];
-      // (F.f)Phi: [Fz p1 + a p0, conj(a) p1 + a pm, conj(a) p0 - Fz pm]
+      const W c0r = c0 * rho, cz = c1 * Fz, cax = c1 * ax, cay = c1 * ay;
+      // c1 (F.f)Phi: c1 [Fz p1 + a p0, conj(a) p1 + a pm, conj(a) p0 - Fz pm]
       W fr[3], fi[3];
-      fr[0] = Fz * u[0].x + (ax * u[1].x - ay * u[1].y);
-      fi[0] = Fz * u[0].y + (ax * u[1].y + ay * u[1].x);
-      fr[1] = (ax * u[0].x + ay * u[0].y) + (ax * u[2].x - ay * u[2].y);
-      fi[1] = (ax * u[0].y - ay * u[0].x) + (ax * u[2].y + ay * u[2].x);
-      fr[2] = (ax * u[1].x + ay * u[1].y) - Fz * u[2].x;
-      fi[2] = (ax * u[1].y - ay * u[1].x) - Fz * u[2].y;
-      W q = (W)0;
+      fr[0] = cz * u[0].x + (cax * u[1].x - cay * u[1].y);
+      fi[0] = cz * u[0].y + (cax * u[1].y + cay * u[1].x);
+      fr[1] = (cax * u[0].x + cay * u[0].y) + (cax * u[2].x - cay * u[2].y);
+      fi[1] = (cax * u[0].y - cay * u[0].x) + (cax * u[2].y + cay * u[2].x);
+      fr[2] = (cax * u[1].x + cay * u[1].y) - cz * u[2].x;
+      fi[2] = (cax * u[1].y - cay * u[1].x) - cz * u[2].y;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        q += u[c].x * lin_r[c] + u[c].y * lin_i[c];
-        const W hr = lin_r[c] + c0 * rho * u[c].x + c1 * fr[c];
-        const W hi = lin_i[c] + c0 * rho * u[c].y + c1 * fi[c];
-        A.out0[sbase + c * npts + off] = mk<C>(hr, hi);
+        acc[0] += u[c].x * lin_r[c] + u[c].y * lin_i[c];
+        A.out0[at + c * npts] = mk<C>(lin_r[c] + (c0r * u[c].x + fr[c]), lin_i[c] + (c0r * u[c].y + fi[c]));
         acc[3 + c] += V * m[c];
         acc[6 + c] += rho * m[c];
         acc[9 + c] += m[c];
       }
-      acc[0] += q;
       acc[1] += rho * rho;
       acc[2] += (W)2 * (ax * ax + ay * ay) + Fz * Fz;
     } else {  // ROW_INV_P: step-model reductions (Eqs. an, bn and the sin/cos form of E(theta))
-      C f[3], h[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) { f[c] = A.in3[sbase + c * npts + off]; h[c] = A.in4[sbase + c * npts + off]; }
       if constexpr (MODE == ROW_INV_P_HY) {
-        // H_lin P kept for the update of H_lin Phi by linearity; the radial part of P
-        // in FP64 (P's FP32 values against the FP64 Phi) for the exact tangent correction
+        // H_lin P kept for the update of H_lin Phi by linearity; the radial part of P (P's FP32
+        // values against the FP64 Phi) and ||P||^2 to double-word accuracy for the exact tangent
+        // correction and the normalisation of the step
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          A.out0[sbase + c * npts + off] = mk<C>(lin_r[c], lin_i[c]);
-          const double2 g = A.phi64[sbase + c * npts + off];
-          const double ux = (double)u[c].x, uy = (double)u[c].y;
-          rphi += g.x * ux + g.y * uy;
-          pp64 += ux * ux + uy * uy;
+          A.out0[at + c * npts] = mk<C>(lin_r[c], lin_i[c]);
+          dwa_mulf(rphi, dw_of(g64[c].x), u[c].x);
+          dwa_mulf(rphi, dw_of(g64[c].y), u[c].y);
+          dwa_sq(pp, u[c].x);
+          dwa_sq(pp, u[c].y);
         }
       }
       W hpp = (W)0, hphip = (W)0, Rv = (W)0, rf = (W)0, rp = (W)0;
@@ -427,76 +466,72 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
         rf += f[c].x * f[c].x + f[c].y * f[c].y;
         rp += u[c].x * u[c].x + u[c].y * u[c].y;
       }
-      // spin vectors F(Phi), F(P) and the symmetric cross term Re F~(Phi, P)
-      const W s2 = (W)1.4142135623730951;
+      // spin vectors F(Phi), F(P) and the symmetric cross term Re F~(Phi, P), through
+      // a(Phi + e P) = a(Phi) + e (a1 + a2) + e^2 a(P); Re F~ is half the e coefficient of F:
+      // F_xy . G_xy = 2 Re(conj(a_F) a_G)
       W aFx, aFy, aPx, aPy, a1x, a1y, a2x, a2y;
       spin_a<W>(f[0], f[1], f[2], aFx, aFy);
       spin_a<W>(u[0], u[1], u[2], aPx, aPy);
-      // a(Phi + e P) = a(Phi) + e (a1 + a2) + e^2 a(P); Re F~ is half the e coefficient of F
       spin_a<W>(f[0], u[1], f[2], a1x, a1y);
       spin_a<W>(u[0], f[1], u[2], a2x, a2y);
-      const W FFx = s2 * aFx, FFy = -s2 * aFy;
+      const W aXx = a1x + a2x, aXy = a1y + a2y;    // twice the cross term's a
       const W FFz = (f[0].x * f[0].x + f[0].y * f[0].y) - (f[2].x * f[2].x + f[2].y * f[2].y);
-      const W FPx = s2 * aPx, FPy = -s2 * aPy;
       const W FPz = (u[0].x * u[0].x + u[0].y * u[0].y) - (u[2].x * u[2].x + u[2].y * u[2].y);
-      const W FXx = (W)0.5 * s2 * (a1x + a2x), FXy = -(W)0.5 * s2 * (a1y + a2y);
       const W FXz = (f[0].x * u[0].x + f[0].y * u[0].y) - (f[2].x * u[2].x + f[2].y * u[2].y);
       acc[0] += hpp;
       acc[1] += hphip;
-      acc[2] += Rv;
-      acc[3] += rf * Rv;
-      acc[4] += rf * rp;
-      acc[5] += Rv * Rv;
-      acc[6] += Rv * rp;
-      acc[7] += rp * rp;
-      acc[8] += FFx * FXx + FFy * FXy + FFz * FXz;
-      acc[9] += FFx * FPx + FFy * FPy + FFz * FPz;
-      acc[10] += FXx * FXx + FXy * FXy + FXz * FXz;
-      acc[11] += FXx * FPx + FXy * FPy + FXz * FPz;
-      acc[12] += FPx * FPx + FPy * FPy + FPz * FPz;
+      if (MODE == ROW_INV_P) accR += Rv;
+      acc[2] += rf * Rv;
+      acc[3] += rf * rp;
+      acc[4] += Rv * Rv;
+      acc[5] += Rv * rp;
+      acc[6] += rp * rp;
+      acc[7] += (aFx * aXx + aFy * aXy) + FFz * FXz;
+      acc[8] += (W)2 * (aFx * aPx + aFy * aPy) + FFz * FPz;
+      acc[9] += (W)0.5 * (aXx * aXx + aXy * aXy) + FXz * FXz;
+      acc[10] += (aXx * aPx + aXy * aPy) + FXz * FPz;
+      acc[11] += (W)2 * (aPx * aPx + aPy * aPy) + FPz * FPz;
     }
   }
   if (MODE == ROW_INV_LIN) return;
-  const bool mx[13] = {};
+  const bool mx[14] = {};
   if (MODE == ROW_INV_H) {
-    const W a12[12] = {acc[0], acc[1], acc[2], acc[3], acc[4], acc[5], acc[6], acc[7], acc[8], acc[9], acc[10], acc[11]};
     const bool mx12[12] = {};
     const int slots[12] = {SL_Q, SL_RHO2, SL_F2, SL_V0, SL_V1, SL_V2, SL_C0, SL_C1, SL_C2, SL_M0, SL_M1, SL_M2};
-    store_partials<12, W>(a12, slots, mx12, red, A.part, sslot, A.pmax, rb);
+    store_partials<12, W>(acc, slots, mx12, red, A.part, sslot, A.pmax, rb);
     if (A.fuse && last_block(A.cnt, s, bps, &last_flag)) sc_obs<PV>(A.sc, s, tail);
   } else {
-    const int slots[13] = {SL_HPP, SL_HPHIP, SL_RPHI, SL_IFR, SL_IFP, SL_IRR, SL_IRP, SL_IPP,
-                           SL_JFR, SL_JFP, SL_JRR, SL_JRP, SL_JPP};
-    store_partials<13, W>(acc, slots, mx, red, A.part, sslot, A.pmax, rb);
+    const int slots[14] = {SL_HPP, SL_HPHIP, SL_IFR, SL_IFP, SL_IRR, SL_IRP, SL_IPP,
+                           SL_JFR, SL_JFP, SL_JRR, SL_JRP, SL_JPP, SL_RPHI, SL_P2};
     if constexpr (MODE == ROW_INV_P_HY) {
-      // the normalisation of the step needs these two to FP64 accuracy
-      double v2[2] = {rphi, pp64};
-      const bool mx2[2] = {false, false};
-      block_reduce<2>(v2, red, mx2);
-      const int slots2[2] = {SL_RPHI, SL_P2};
-      __syncthreads();   // thread 0 of store_partials wrote SL_RPHI's FP32 sum before
-      put_partials<2>(A.part, sslot, A.pmax, rb, slots2, v2, mx2, true);
+      DF all[14];
+#pragma unroll
+      for (int k = 0; k < 12; ++k) all[k] = DF{acc[k], 0.0f};
+      all[12] = dwa_value(rphi);
+      all[13] = dwa_value(pp);
+      double v[14];
+      block_reduce_dw<14>(all, v, red);
+      put_partials<14>(A.part, sslot, A.pmax, rb, slots, v, mx, true);
+    } else {
+      W a13[13];
+      int s13[13];
+      const bool m13[13] = {};
+#pragma unroll
+      for (int k = 0; k < 13; ++k) { a13[k] = k < 12 ? acc[k] : accR; s13[k] = slots[k]; }
+      store_partials<13, W>(a13, s13, m13, red, A.part, sslot, A.pmax, rb);
     }
     if (A.fuse && last_block(A.cnt, s, bps, &last_flag)) sc_step<PV>(A.sc, s, tail);
   }
 }
 
+// Blocks of kThreads per SM each pass is compiled for: 3 (at most 56 registers, six 192-thread tiles per
+// SM; the passes with fused sums spill a few values) for FP32, 2 (84 registers, four tiles) for FP64 and for
+// the last pass of a hybrid iteration, whose Algorithm 2 step alone would take 113 for its grid sums.
 template <class T, int MODE>
-__global__ void __launch_bounds__(kThreads) k_row(ChainArgs<T> A, int R, int ept) {
+constexpr int row_blocks() { return sizeof(T) == 4 && MODE != ROW_INV_P_HY ? 3 : 2; }
+template <class T, int MODE>
+__global__ void __launch_bounds__(kThreads, row_blocks<T, MODE>()) k_row(ChainArgs<T> A, int R, int ept) {
   row_pass<T, MODE>(A, R, ept);
-}
-
-// The FP32 inverse passes with fused reductions (the heaviest epilogues) are
-// compiled for three blocks of kThreads per SM (at most 56 registers, a few values
-// spilled): six 192-thread tiles per SM instead of four.
-template <class T, int MODE>
-__global__ void __launch_bounds__(kThreads, 3) k_row_lean(ChainArgs<T> A, int R, int ept) {
-  row_pass<T, MODE>(A, R, ept);
-}
-
-template <class T, int MODE>
-constexpr bool row_lean() {
-  return sizeof(T) == 4 && (MODE == ROW_INV_H || MODE == ROW_INV_P || MODE == ROW_INV_PRE);
 }
 
 // ============================================================== column passes (y or z axis)
@@ -513,66 +548,71 @@ __global__ void __launch_bounds__(kThreads) k_col(ChainArgs<T> A, int axis, int 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int na = A.g.n[axis], La = A.g.log2n[axis];
   const long long npts = A.g.npts;
-  const int ni = (axis == 1) ? A.g.n[0] : A.g.n[0] * A.g.n[1];   // inner (faster) extent
-  const int no = (int)(npts / ((long long)na * ni));             // outer (slower) extent
-  const int tpo = ni / TC;                                       // tiles per outer index
-  const int bps = tpo * no;
+  const int Li = (axis == 1) ? A.g.log2n[0] : A.g.log2n[0] + A.g.log2n[1];   // log2 of the inner (faster) extent
+  const int LT = __ffs(TC) - 1;
+  const int Lt = Li - LT;                                        // log2 of the tiles per outer index
+  const int bps = (int)(npts >> (La + LT));
   const int s = blockIdx.x / bps;
-  const int tb = blockIdx.x % bps;
-  C* s_tw = (C*)smem_raw;
-  load_tw<T>(s_tw, A.tw[axis], na, ept);   // constant table: before the wait on the previous kernel
+  const int tb = blockIdx.x - s * bps;
   pdl_wait();
   if (s >= A.nsolve || !gate_ok(A.st, A.gate, s)) return;
-  const int o = tb / tpo;
-  const int i0 = (tb % tpo) * TC;
+  C* s_tw = (C*)smem_raw;
+  const int o = tb >> Lt;
+  const int i0 = (tb - (o << Lt)) << LT;
   const int b0 = fft_padded_len<C>(na);   // the lines lie behind the table
   C* buf = s_tw + b0;
-  const int per = na * TC;
   const int NPL = col_line_len<C>(na, TC);        // padded line length
   const int CS = TC * NPL;                     // component stride in smem
   C* buf2 = buf + 3 * CS;            // second 3-component tile (YMID_H, YINV_H)
   double* red = (double*)(buf2 + 3 * CS);
-  const long long sbase = (long long)s * 3 * npts;
-  const long long obase = (long long)o * na * ni + i0;
   const SolveState& S = A.st[s];
-  const PhysDev ph = A.phys[s];
+  const PhysDev& ph = A.phys[s];
   const W piA = geo_piL<W>(A.g, axis);
   const int nx = A.g.n[0];
-  // smem index of element j of column t, component c: c * CS + t * NPL + pad(j)
-  auto sidx = [&](int c, int t, int j) { return c * CS + t * NPL + fft_pad<C>(j); };
+  // a thread stays on one column of the tile (the block is a multiple of TC threads): column t, from
+  // row j0 in steps of dj; its first point, and element j of component c in shared memory
+  const int t = threadIdx.x & (TC - 1), j0 = threadIdx.x >> LT, dj = blockDim.x >> LT;
+  const long long col = (long long)s * 3 * npts + ((long long)o << (La + Li)) + i0 + t;
+  const int lt = t * NPL;
+  auto sidx = [&](int c, int j) { return c * CS + lt + fft_pad<C>(j); };
 
-  // load the in0 tile (and in1 for YINV_H) in natural order; global reads coalesced over t
-  for (int e = threadIdx.x; e < per; e += blockDim.x) {
-    const int j = e / TC, t = e - j * TC;
+  // the in0 tile (and in1 for YINV_H) in natural order, by asynchronous copies that are under way
+  // while the twiddle table is set up
+  for (int j = j0; j < na; j += dj) {
+    const long long at = col + ((long long)j << Li);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const C v = A.in0[sbase + c * npts + obase + (long long)j * ni + t];
-      buf[sidx(c, t, j)] = (MODE == COL_INV || MODE == COL_YINV_H) ? swp(v) : v;
-      if (MODE == COL_YINV_H) buf2[sidx(c, t, j)] = A.in1[sbase + c * npts + obase + (long long)j * ni + t];
+      copy_async(&buf[sidx(c, j)], A.in0 + at + c * npts);
+      if (MODE == COL_YINV_H) copy_async(&buf2[sidx(c, j)], A.in1 + at + c * npts);
     }
   }
-  __syncthreads();
-
-  // inner index -> (kx [, ky]) wavenumbers (inputs are spectral along the faster axes)
-  auto kinner = [&](int t, W& kx, W& ky) {
+  load_tw<T>(s_tw, A.tw[axis], na, ept);
+  // wavenumbers of the column's inner index (the inputs are spectral along the faster axes)
+  W kx, kyc;
+  {
     const int ii = i0 + t;
-    if (axis == 1) { kx = wavenum<W>(ii, nx, geo_piL<W>(A.g, 0)); ky = (W)0; }
-    else { kx = wavenum<W>(ii % nx, nx, geo_piL<W>(A.g, 0)); ky = wavenum<W>(ii / nx, A.g.n[1], geo_piL<W>(A.g, 1)); }
-  };
+    kx = wavenum<W>(ii & (nx - 1), nx, geo_piL<W>(A.g, 0));
+    kyc = axis == 1 ? (W)0 : wavenum<W>(ii >> A.g.log2n[0], A.g.n[1], geo_piL<W>(A.g, 1));
+  }
+  const W k2c = (W)0.5 * (kx * kx + kyc * kyc);
+  const W Om = pick<W>(ph.Omega, ph.fOmega), g = pick<W>(ph.gamma, ph.fgamma);
+  const W al[3] = {pick<W>(S.alpha[0], S.falpha[0]), pick<W>(S.alpha[1], S.falpha[1]), pick<W>(S.alpha[2], S.falpha[2])};
+  copy_wait();
+  __syncthreads();
 
   W acc[3] = {(W)0, (W)0, (W)0};
   // one transform, or (the middle passes) a forward one, the work in k and the inverse one: a loop
-  // around one inlined copy of the transforms
+  // around one inlined copy of the transforms.  The inverse transforms are forward ones whose values
+  // are read at index -j
   constexpr bool middle = (MODE == COL_MID_H || MODE == COL_MID_PRE || MODE == COL_YMID_H || MODE == COL_YINV_H);
 #pragma unroll 1
   for (int phase = 0; phase < (middle ? 2 : 1); ++phase) {
     if (MODE == COL_YINV_H && phase == 1) {
       // buf2: A -> F_y A, times v_y; then F_y^-1 of both: buf from C, buf2 -> G
-      for (int e = threadIdx.x; e < per; e += blockDim.x) {
-        const int j = e / TC, t = e - j * TC;
+      for (int j = j0; j < na; j += dj) {
         const W vy = wavenum<W>(j, na, piA);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) buf2[sidx(c, t, j)] = swp(cscale(buf2[sidx(c, t, j)], vy));
+        for (int c = 0; c < 3; ++c) buf2[sidx(c, j)] = cscale(buf2[sidx(c, j)], vy);
       }
       __syncthreads();
     } else if (phase == 1) {
@@ -581,28 +621,29 @@ __global__ void __launch_bounds__(kThreads) k_col(ChainArgs<T> A, int axis, int 
         // of Phi by the step applied this iteration (Phi_hat <- g (c Phi_hat + t P_hat_prev)),
         // keep this P_hat, and sum 1/2 |k|^2 |Phi_hat_l|^2 and 1/2 |k|^2 Re(Phi_hat_l conj P_hat_l)
         const bool upd = A.khat_upd && S.upd_applied;
-        const W uc = pick<W>(S.upd_c, S.fupd_c), us = pick<W>(S.upd_s, S.fupd_s), usc = pick<W>(S.upd_scale, S.fupd_scale);
+        const W usc = pick<W>(S.upd_scale, S.fupd_scale);
+        const W uc = usc * pick<W>(S.upd_c, S.fupd_c), us = usc * pick<W>(S.upd_s, S.fupd_s);
         W kacc[6] = {(W)0, (W)0, (W)0, (W)0, (W)0, (W)0};
-        for (int e = threadIdx.x; e < per; e += blockDim.x) {
-          const int j = e / TC, t = e - j * TC;
-          W kx, ky, kz = (W)0;
-          kinner(t, kx, ky);
-          if (axis == 1) ky = wavenum<W>(j, na, piA);
-          else kz = wavenum<W>(j, na, piA);
-          const W k2h = (W)0.5 * (kx * kx + ky * ky + kz * kz);
-          const long long gi = sbase + obase + (long long)j * ni + t;
+        for (int j = j0; j < na; j += dj) {
+          const W ka = wavenum<W>(j, na, piA);
+          const W k2h = k2c + (W)0.5 * ka * ka;
+          const long long at = col + ((long long)j << Li);
+          C xv[3], po[3];
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
-            const C pv = buf[sidx(c, t, j)];
-            C xv = A.xhat[gi + c * npts];
+            xv[c] = A.xhat[at + c * npts];
+            if (upd) po[c] = A.phat[at + c * npts];
+          }
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const C pv = buf[sidx(c, j)];
             if (upd) {
-              const C po = A.phat[gi + c * npts];
-              xv = mk<C>(usc * (uc * xv.x + us * po.x), usc * (uc * xv.y + us * po.y));
-              A.xhat[gi + c * npts] = xv;
+              xv[c] = mk<C>(uc * xv[c].x + us * po[c].x, uc * xv[c].y + us * po[c].y);
+              A.xhat[at + c * npts] = xv[c];
             }
-            A.phat[gi + c * npts] = pv;
-            kacc[c] += k2h * (xv.x * xv.x + xv.y * xv.y);
-            kacc[3 + c] += k2h * (xv.x * pv.x + xv.y * pv.y);
+            A.phat[at + c * npts] = pv;
+            kacc[c] += k2h * (xv[c].x * xv[c].x + xv[c].y * xv[c].y);
+            kacc[3 + c] += k2h * (xv[c].x * pv.x + xv[c].y * pv.y);
           }
         }
         const bool kmx[6] = {false, false, false, false, false, false};
@@ -611,18 +652,13 @@ __global__ void __launch_bounds__(kThreads) k_col(ChainArgs<T> A, int axis, int 
       }
 
       // pointwise in k: the kinetic + SOC symbol (H chains) or the kinetic preconditioner; with
-      // YMID_H also G_c = F_y^-1[v_y F_y A_c] in buf2.  Results go back exchanged (inverse transform)
-      const W al[3] = {pick<W>(S.alpha[0], S.falpha[0]), pick<W>(S.alpha[1], S.falpha[1]), pick<W>(S.alpha[2], S.falpha[2])};
-      const W g = pick<W>(ph.gamma, ph.fgamma);
+      // YMID_H also G_c = F_y^-1[v_y F_y A_c] in buf2
       const bool use_pd = (A.sc.opts.precond == GPSOC_PRECOND_COMBINED || A.sc.opts.precond == GPSOC_PRECOND_KINETIC);
-      for (int e = threadIdx.x; e < per; e += blockDim.x) {
-        const int j = e / TC, t = e - j * TC;
-        const int i1 = sidx(0, t, j), i2 = sidx(1, t, j), i3 = sidx(2, t, j);
-        W kx, ky, kz = (W)0;
-        kinner(t, kx, ky);
-        if (axis == 1) ky = wavenum<W>(j, na, piA);
-        else kz = wavenum<W>(j, na, piA);
-        const W k2h = (W)0.5 * (kx * kx + ky * ky + kz * kz);
+      const W gx = g * kx;
+      for (int j = j0; j < na; j += dj) {
+        const int i1 = sidx(0, j), i2 = sidx(1, j), i3 = sidx(2, j);
+        const W ka = wavenum<W>(j, na, piA);
+        const W k2h = k2c + (W)0.5 * ka * ka;
         if (MODE == COL_MID_PRE) {
           // P_Delta (Eq. PreCondKin); the potential-only and no-preconditioner variants keep
           // the coefficients (the transform pair is then the identity up to rounding)
@@ -633,35 +669,28 @@ __global__ void __launch_bounds__(kThreads) k_col(ChainArgs<T> A, int axis, int 
             const W d01 = d0 * d1;
             const W inv = (W)1 / (d01 * d2);
             const W r01 = d2 * inv;
-            buf[i1] = swp(cscale(buf[i1], d1 * r01));
-            buf[i2] = swp(cscale(buf[i2], d0 * r01));
-            buf[i3] = swp(cscale(buf[i3], d01 * inv));
-          } else {
-            buf[i1] = swp(buf[i1]);
-            buf[i2] = swp(buf[i2]);
-            buf[i3] = swp(buf[i3]);
+            buf[i1] = cscale(buf[i1], d1 * r01);
+            buf[i2] = cscale(buf[i2], d0 * r01);
+            buf[i3] = cscale(buf[i3], d01 * inv);
           }
         } else {
           const C p1 = buf[i1], p0 = buf[i2], pm = buf[i3];
           if (MODE == COL_YMID_H) {
-            buf2[i1] = swp(cscale(p1, ky));
-            buf2[i2] = swp(cscale(p0, ky));
-            buf2[i3] = swp(cscale(pm, ky));
+            buf2[i1] = cscale(p1, ka);
+            buf2[i2] = cscale(p0, ka);
+            buf2[i3] = cscale(pm, ka);
           }
           // kinetic per component (Parseval): sum 1/2 |k|^2 |phat_l|^2
           acc[0] += k2h * (p1.x * p1.x + p1.y * p1.y);
           acc[1] += k2h * (p0.x * p0.x + p0.y * p0.y);
           acc[2] += k2h * (pm.x * pm.x + pm.y * pm.y);
-          // -gamma S symbol: s0 = -kx + i ky (L0), s1 = -(kx + i ky) (L1)
+          // -gamma S symbol with -s0 = kx - i ky (L0), -s1 = kx + i ky (L1):
           // out_1 = K p1 - g s0 p0 ; out_0 = K p0 - g (s1 p1 + s0 pm) ; out_-1 = K pm - g s1 p0
-          const W s0r = -kx, s0i = ky, s1r = -kx, s1i = -ky;
-          const W a_r = s0r * p0.x - s0i * p0.y, a_i = s0r * p0.y + s0i * p0.x;   // s0 p0
-          const W b_r = s1r * p1.x - s1i * p1.y, b_i = s1r * p1.y + s1i * p1.x;   // s1 p1
-          const W c_r = s0r * pm.x - s0i * pm.y, c_i = s0r * pm.y + s0i * pm.x;   // s0 pm
-          const W d_r = s1r * p0.x - s1i * p0.y, d_i = s1r * p0.y + s1i * p0.x;   // s1 p0
-          buf[i1] = mk<C>(k2h * p1.y - g * a_i, k2h * p1.x - g * a_r);
-          buf[i2] = mk<C>(k2h * p0.y - g * (b_i + c_i), k2h * p0.x - g * (b_r + c_r));
-          buf[i3] = mk<C>(k2h * pm.y - g * d_i, k2h * pm.x - g * d_r);
+          const W gy = g * (axis == 1 ? ka : kyc);
+          const W sx = p1.x + pm.x, sy = p1.y + pm.y, dx = p1.x - pm.x, dy = p1.y - pm.y;
+          buf[i1] = mk<C>(k2h * p1.x + (gx * p0.x + gy * p0.y), k2h * p1.y + (gx * p0.y - gy * p0.x));
+          buf[i2] = mk<C>(k2h * p0.x + (gx * sx - gy * dy), k2h * p0.y + (gx * sy + gy * dx));
+          buf[i3] = mk<C>(k2h * pm.x + (gx * p0.x - gy * p0.y), k2h * pm.y + (gx * p0.y + gy * p0.x));
         }
       }
       __syncthreads();
@@ -672,68 +701,30 @@ __global__ void __launch_bounds__(kThreads) k_col(ChainArgs<T> A, int axis, int 
     fft_lines<C, true>(first, lines, NPL, La, ept);
   }
 
-  if (MODE == COL_FWD) {
-    for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int j = e / TC, t = e - j * TC;
+  const W sc = (MODE == COL_INV) ? (W)A.scale : (W)1;
+  // 2D: T' = F_y^-1[M F_y A] + ny Omega y v_x A; 3D: the factors of the axes transformed so far
+  const W nz = (W)A.g.n[2];
+  const W rx = (W)A.g.n[1] * (MODE == COL_YINV_H ? nz : (W)1) * Om * kx;
+  for (int j = j0; j < na; j += dj) {
+    const long long at = col + ((long long)j << Li);
+    const int jr = (MODE == COL_FWD) ? j : (-j & (na - 1));
+    if (MODE == COL_YMID_H || MODE == COL_YINV_H) {
+      const W rot = rx * coord<W>(A.g, 1, j);
+      C a[3];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) A.out0[sbase + c * npts + obase + (long long)j * ni + t] = buf[sidx(c, t, j)];
-    }
-    return;
-  }
-  if (MODE == COL_INV) {
-    const W sc = (W)A.scale;
-    for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int j = e / TC, t = e - j * TC;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const C v = swp(buf[sidx(c, t, j)]);
-        A.out0[sbase + c * npts + obase + (long long)j * ni + t] = mk<C>(v.x * sc, v.y * sc);
-      }
-    }
-    return;
-  }
-  if (MODE == COL_YINV_H) {
-    const W nfac = (W)A.g.n[1] * (W)A.g.n[2];  // ny * nz
-    const W nz = (W)A.g.n[2];
-    for (int e = threadIdx.x; e < per; e += blockDim.x) {
-      const int j = e / TC, t = e - j * TC;
-      W kx, ky;
-      kinner(t, kx, ky);
-      const W y = coord<W>(A.g, 1, j);
-      const W rot = nfac * pick<W>(ph.Omega, ph.fOmega) * y * kx;
-      const long long gi = sbase + obase + (long long)j * ni + t;
+      for (int c = 0; c < 3; ++c) a[c] = __ldg((MODE == COL_YINV_H ? A.in1 : A.in0) + at + c * npts);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const C a = A.in1[gi + c * npts];
-        const C cv = swp(buf[sidx(c, t, j)]);
-        A.out0[gi + c * npts] = mk<C>(cv.x + rot * a.x, cv.y + rot * a.y);
-        const C gv = swp(buf2[sidx(c, t, j)]);
-        A.out1[gi + c * npts] = mk<C>(gv.x * nz, gv.y * nz);
-      }
-    }
-    return;
-  }
-
-  const W nrot = (W)A.g.n[1];  // 2D: T' = F_y^-1[M F_y A] + ny Omega y v_x A
-  const W Om = pick<W>(ph.Omega, ph.fOmega);
-  for (int e = threadIdx.x; e < per; e += blockDim.x) {
-    const int j = e / TC, t = e - j * TC;
-    const long long gi = sbase + obase + (long long)j * ni + t;
-    if (MODE == COL_YMID_H) {
-      W kx, ky;
-      kinner(t, kx, ky);
-      const W y = coord<W>(A.g, 1, j);
-      const W rot = nrot * Om * y * kx;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const C a = A.in0[gi + c * npts];
-        const C v = swp(buf[sidx(c, t, j)]);
-        A.out0[gi + c * npts] = mk<C>(v.x + rot * a.x, v.y + rot * a.y);
-        A.out1[gi + c * npts] = swp(buf2[sidx(c, t, j)]);
+        const C v = buf[sidx(c, jr)], gv = buf2[sidx(c, jr)];
+        A.out0[at + c * npts] = mk<C>(v.x + rot * a[c].x, v.y + rot * a[c].y);
+        A.out1[at + c * npts] = (MODE == COL_YINV_H) ? mk<C>(gv.x * nz, gv.y * nz) : gv;
       }
     } else {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) A.out0[gi + c * npts] = swp(buf[sidx(c, t, j)]);
+      for (int c = 0; c < 3; ++c) {
+        const C v = buf[sidx(c, jr)];
+        A.out0[at + c * npts] = (MODE == COL_INV) ? mk<C>(v.x * sc, v.y * sc) : v;
+      }
     }
   }
   if (MODE == COL_MID_H || MODE == COL_YMID_H) {
@@ -944,10 +935,7 @@ static void row_go(const ChainArgs<T>& a, cudaStream_t st) {
   const size_t sm = row_smem<T>(a.g, MODE, a.nsolve);
   const int ept = row_ept<T>(a.g, a.nsolve);
   const int threads = round_threads(3 * R * a.g.n[0] / ept);
-  if constexpr (row_lean<T, MODE>())
-    launch_pdl(k_row_lean<T, MODE>, nb, threads, sm, st, a, R, ept);
-  else
-    launch_pdl(k_row<T, MODE>, nb, threads, sm, st, a, R, ept);
+  launch_pdl(k_row<T, MODE>, nb, threads, sm, st, a, R, ept);
 }
 
 template <class T>
@@ -962,8 +950,8 @@ void launch_row(int mode, const ChainArgs<T>& a, int, const Launch&, cudaStream_
     case ROW_INV_PLAIN: row_go<T, ROW_INV_PLAIN>(a, st); break;
     case ROW_INV_LIN: row_go<T, ROW_INV_LIN>(a, st); break;
     case ROW_FWD_UPD: row_go<T, ROW_FWD_UPD>(a, st); break;
-    case ROW_FWD_PRE_HY: row_go<T, ROW_FWD_PRE_HY>(a, st); break;
-    case ROW_INV_P_HY: row_go<T, ROW_INV_P_HY>(a, st); break;
+    case ROW_FWD_PRE_HY: if constexpr (sizeof(T) == 4) row_go<T, ROW_FWD_PRE_HY>(a, st); break;
+    case ROW_INV_P_HY: if constexpr (sizeof(T) == 4) row_go<T, ROW_INV_P_HY>(a, st); break;
   }
 }
 
@@ -997,11 +985,10 @@ cudaError_t chain_prepare() {
   GPSOC_ATTR((k_row<T, ROW_FWD_PLAIN>)) GPSOC_ATTR((k_row<T, ROW_FWD_PROJ>)) GPSOC_ATTR((k_row<T, ROW_FWD_PRE>))
   GPSOC_ATTR((k_row<T, ROW_INV_H>)) GPSOC_ATTR((k_row<T, ROW_INV_P>)) GPSOC_ATTR((k_row<T, ROW_INV_PRE>))
   GPSOC_ATTR((k_row<T, ROW_INV_PLAIN>)) GPSOC_ATTR((k_row<T, ROW_INV_LIN>)) GPSOC_ATTR((k_row<T, ROW_FWD_UPD>))
-  GPSOC_ATTR((k_row<T, ROW_FWD_PRE_HY>)) GPSOC_ATTR((k_row<T, ROW_INV_P_HY>))
   GPSOC_ATTR((k_col<T, COL_FWD>)) GPSOC_ATTR((k_col<T, COL_INV>)) GPSOC_ATTR((k_col<T, COL_MID_H>))
   GPSOC_ATTR((k_col<T, COL_MID_PRE>)) GPSOC_ATTR((k_col<T, COL_YMID_H>)) GPSOC_ATTR((k_col<T, COL_YINV_H>))
   if constexpr (sizeof(T) == 4) {
-    GPSOC_ATTR((k_row_lean<T, ROW_INV_H>)) GPSOC_ATTR((k_row_lean<T, ROW_INV_P>)) GPSOC_ATTR((k_row_lean<T, ROW_INV_PRE>))
+    GPSOC_ATTR((k_row<T, ROW_FWD_PRE_HY>)) GPSOC_ATTR((k_row<T, ROW_INV_P_HY>))
   }
 #undef GPSOC_ATTR
   return e;

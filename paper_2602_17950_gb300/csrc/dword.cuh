@@ -190,6 +190,60 @@ GPSOC_DW DF dw_of(double x) {
   }
   return r;
 }
+// binary64 -> binary32 by integer operations (the high word of dw_of: half-ulp ties up, values
+// below 2^-126 become signed zeros)
+GPSOC_DW float narrow_f(double x) {
+  const unsigned H = d_hi(x), L = d_lo(x);
+  const unsigned sign = H & 0x80000000u;
+  const int E = (int)((H >> 20) & 0x7ffu);
+  unsigned u = (sign | ((unsigned)(E - 896) << 23) | ((H & 0xfffffu) << 3) | (L >> 29)) + ((L >> 28) & 1u);
+  if (E < 897) u = sign;
+  if (E > 1150) u = (E == 2047 && ((H & 0xfffffu) | L) != 0u) ? 0x7fc00000u : (sign | 0x7f800000u);
+  return f_from(u);
+}
+// Running sums of products in a double word that is normalised once, at the end (dwa_value): the high
+// word takes each product's leading part exactly (TwoSum), the low word the parts it leaves and the
+// products' own error terms.  Relative to the sum of the terms' moduli the error is a few u^2 as with
+// dw_add and dw_mul for every term, at 9 to 12 instructions a term instead of 28.
+GPSOC_DW void dwa_add(DF& A, float p, float e) {
+  const DF s = dw_two_sum(A.hi, p);
+  A.hi = s.hi;
+  A.lo = rn_add(A.lo, rn_add(s.lo, e));
+}
+GPSOC_DW void dwa_sq(DF& A, float a) {               // += a a
+  const float p = rn_mul(a, a);
+  dwa_add(A, p, rn_fma(a, a, -p));
+}
+GPSOC_DW void dwa_mulf(DF& A, DF a, float b) {       // += a b
+  const float p = rn_mul(a.hi, b);
+  dwa_add(A, p, rn_fma(a.lo, b, rn_fma(a.hi, b, -p)));
+}
+GPSOC_DW void dwa_mul(DF& A, DF a, DF b) {           // += a b
+  const float p = rn_mul(a.hi, b.hi);
+  dwa_add(A, p, rn_fma(a.lo, b.hi, rn_fma(a.hi, b.lo, rn_fma(a.hi, b.hi, -p))));
+}
+GPSOC_DW void dwa_sub(DF& A, DF a, DF b) {           // -= a b
+  const float p = rn_mul(-a.hi, b.hi);
+  dwa_add(A, p, rn_fma(-a.lo, b.hi, rn_fma(-a.hi, b.lo, rn_fma(-a.hi, b.hi, -p))));
+}
+GPSOC_DW void dwa_sqd(DF& A, DF a) {                 // += a a
+  const float p = rn_mul(a.hi, a.hi);
+  dwa_add(A, p, rn_fma(a.hi + a.hi, a.lo, rn_fma(a.hi, a.hi, -p)));
+}
+GPSOC_DW DF dwa_of_mul(DF a, DF b) {                 // a sum that opens with a b
+  DF r;
+  r.hi = rn_mul(a.hi, b.hi);
+  r.lo = rn_fma(a.lo, b.hi, rn_fma(a.hi, b.lo, rn_fma(a.hi, b.hi, -r.hi)));
+  return r;
+}
+GPSOC_DW DF dwa_of_sqd(DF a) {
+  DF r;
+  r.hi = rn_mul(a.hi, a.hi);
+  r.lo = rn_fma(a.hi + a.hi, a.lo, rn_fma(a.hi, a.hi, -r.hi));
+  return r;
+}
+GPSOC_DW DF dwa_value(DF A) { return dw_fast_two_sum(A.hi, A.lo); }
+
 // double word -> binary64, correctly rounded: one FP64 add of the two exact widenings
 GPSOC_DW double dw_to_double(DF a) { return widen_f(a.hi) + widen_f(a.lo); }
 // hi and lo of an FP64 value by FP64 arithmetic, for state fields the double-word

@@ -204,9 +204,8 @@ struct FftPad16 { __device__ __forceinline__ int operator()(int e) const { retur
 // to 256 with 8 elements per thread) its passes need no block barrier, only the warp's; before,
 // each pass waited twice for the whole block (24-27% of the stalls of the 256^2 passes).
 //
-// An inverse transform is the forward one of values with real and imaginary part exchanged,
-// exchanged again (swp below), so that one inlined copy serves every transform of a kernel:
-// unrolled passes are 10 to 20 KB of instructions, run once or twice by a block, and a third of
+// The inverse transform is the forward one read at index -j mod n, so that one inlined copy serves
+// every transform of a kernel: unrolled passes are 10 to 20 KB of instructions, run once or twice by a block, and a third of
 // the stalls of the FP64 column passes was waiting for them (ncu, no_instruction) with three.
 template <class C, int E>
 __device__ __forceinline__ void fft_lines_e(int off, int nlines, int NP, int L) {
@@ -231,14 +230,6 @@ __device__ __forceinline__ void fft_lines_e(int off, int nlines, int NP, int L) 
       stockham_fft<C, E>(p, act, g, L, tw, warp);
   }
   __syncthreads();
-}
-
-// real and imaginary part exchanged
-template <class C> __device__ __forceinline__ C swp(C a) {
-  C r;
-  r.x = a.y;
-  r.y = a.x;
-  return r;
 }
 
 }  // namespace gpsoc

@@ -288,10 +288,19 @@ __device__ __forceinline__ W trap_value(const TrapDev& t, const Geo& g, int ix, 
     v += pick<W>(t.half_g2[2], t.fhalf_g2[2]) * z * z;
     r2 += z * z;
   }
-  v += pick<W>(t.quad, t.fquad) * r2 + pick<W>(t.quart, t.fquart) * r2 * r2;
+  if (t.fquad != 0.0f || t.fquart != 0.0f || t.quad != 0.0 || t.quart != 0.0)
+    v += pick<W>(t.quad, t.fquad) * r2 + pick<W>(t.quart, t.fquart) * r2 * r2;
   if (t.userV) v += (W)t.userV[idx];
   return v;
 }
+
+// asynchronous copy of one complex value into shared memory, and the wait for this thread's copies
+template <class C> __device__ __forceinline__ void copy_async(C* smem, const C* gmem) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
+  if constexpr (sizeof(C) == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(d), "l"(gmem) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" :: "r"(d), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // ------------------------------------------------------------------ block reductions (deterministic)
 // FP64 block reductions in a fixed order.  FP64 issue slots are scarce on this

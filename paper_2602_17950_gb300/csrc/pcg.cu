@@ -167,48 +167,56 @@ __global__ void __launch_bounds__(kHyThreads, kHyBlocksPerSM) k_hy_upd(HyArgs A)
   const DF ucm1 = DF{S.dw_ucm1[0], S.dw_ucm1[1]};
   const PhysDev ph = A.phys[s];
   const DF c0 = DF{ph.fc0, ph.c0lo}, c1 = DF{ph.fc1, ph.c1lo};
-  const int nx = A.g.n[0], ny = A.g.n[1];
+  const int nx = A.g.n[0], ny = A.g.n[1], Lx = A.g.log2n[0], Ly = A.g.log2n[1];
+  const bool dphi = upd && A.sc.opts.stop == GPSOC_STOP_DPHI;   // only the stop1 test reads max |dPhi|
   DF acc[6];
   float acc32[6];
 #pragma unroll
   for (int k = 0; k < 6; ++k) { acc[k] = DF{0.0f, 0.0f}; acc32[k] = 0.0f; }
   float dmax = 0.0f;
   for (long long e = threadIdx.x; e < per; e += blockDim.x) {
-    const long long off = ebase + e;
+    const long long off = ebase + e, at = sbase + off;
     // every load of the point first (one memory round trip), then the arithmetic
     double2 f64[3], h64[3];
     float2 q[3], hq[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const long long i = sbase + c * npts + off;
-      f64[c] = A.phi[i];
-      if (red || rec) h64[c] = A.hl[i];
-      if (upd) q[c] = A.p[i];
-      if (rec) hq[c] = A.hlp[i];
+      f64[c] = A.phi[at + c * npts];
+      if (red || rec) h64[c] = A.hl[at + c * npts];
+      if (upd) q[c] = __ldg(A.p + at + c * npts);
+      if (rec) hq[c] = __ldg(A.hlp + at + c * npts);
     }
     DF fx[3], fy[3], hx[3], hy[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const long long i = sbase + c * npts + off;
       fx[c] = dw_of(f64[c].x);
       fy[c] = dw_of(f64[c].y);
-      if (red && !rec) {
+      if (red || rec) {
         hx[c] = dw_of(h64[c].x);
         hy[c] = dw_of(h64[c].y);
       }
       if (upd) {
         // the accepted step (Eqs. formula-pcg, update) with the exact tangent direction
-        const DF dx = dw_add(dw_mul(ucm1, fx[c]), dw_mulf(ut, q[c].x));
-        const DF dy = dw_add(dw_mul(ucm1, fy[c]), dw_mulf(ut, q[c].y));
-        dmax = fmaxf(dmax, dx.hi * dx.hi + dy.hi * dy.hi);
-        fx[c] = dw_add(fx[c], dx);
-        fy[c] = dw_add(fy[c], dy);
-        A.phi[i] = make_double2(dw_to_double(fx[c]), dw_to_double(fy[c]));
+        if (dphi) {
+          const float dx = ucm1.hi * fx[c].hi + ut.hi * q[c].x, dy = ucm1.hi * fy[c].hi + ut.hi * q[c].y;
+          dmax = fmaxf(dmax, dx * dx + dy * dy);
+        }
+        DF nx_ = dwa_of_mul(ucm1, fx[c]), ny_ = dwa_of_mul(ucm1, fy[c]);
+        dwa_mulf(nx_, ut, q[c].x);
+        dwa_mulf(ny_, ut, q[c].y);
+        dwa_add(nx_, fx[c].hi, fx[c].lo);
+        dwa_add(ny_, fy[c].hi, fy[c].lo);
+        fx[c] = dwa_value(nx_);
+        fy[c] = dwa_value(ny_);
+        A.phi[at + c * npts] = make_double2(dw_to_double(fx[c]), dw_to_double(fy[c]));
         if (rec) {
           // H_lin is linear: H_lin Phi' = g (c H_lin Phi + t H_lin P)
-          hx[c] = dw_add(dw_mul(uc, dw_of(h64[c].x)), dw_mulf(ut, hq[c].x));
-          hy[c] = dw_add(dw_mul(uc, dw_of(h64[c].y)), dw_mulf(ut, hq[c].y));
-          A.hl[i] = make_double2(dw_to_double(hx[c]), dw_to_double(hy[c]));
+          DF gx = dwa_of_mul(uc, hx[c]), gy = dwa_of_mul(uc, hy[c]);
+          dwa_mulf(gx, ut, hq[c].x);
+          dwa_mulf(gy, ut, hq[c].y);
+          hx[c] = dwa_value(gx);
+          hy[c] = dwa_value(gy);
+          A.hl[at + c * npts] = make_double2(dw_to_double(hx[c]), dw_to_double(hy[c]));
         }
       }
     }
@@ -219,39 +227,58 @@ __global__ void __launch_bounds__(kHyThreads, kHyBlocksPerSM) k_hy_upd(HyArgs A)
     float mf[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      m[c] = dw_add(dw_mul(fx[c], fx[c]), dw_mul(fy[c], fy[c]));
-      acc[0] = dw_add(acc[0], dw_add(dw_mul(fx[c], hx[c]), dw_mul(fy[c], hy[c])));
-      A.phi32[sbase + c * npts + off] = make_float2(fx[c].hi, fy[c].hi);
+      DF t = dwa_of_sqd(fx[c]);
+      dwa_sqd(t, fy[c]);
+      m[c] = dwa_value(t);
+      dwa_mul(acc[0], fx[c], hx[c]);
+      dwa_mul(acc[0], fy[c], hy[c]);
+      dwa_add(acc[3 + c], m[c].hi, m[c].lo);
+      A.phi32[at + c * npts] = make_float2(fx[c].hi, fy[c].hi);
       mf[c] = fx[c].hi * fx[c].hi + fy[c].hi * fy[c].hi;   // the alpha pieces (FP32)
     }
-    const DF rho = dw_add(dw_add(m[0], m[1]), m[2]);
+    DF rho = m[0];
+    dwa_add(rho, m[1].hi, m[1].lo);
+    dwa_add(rho, m[2].hi, m[2].lo);
+    rho = dwa_value(rho);
     // a = phi_1 conj(phi_0) + phi_0 conj(phi_-1) (components ordered 1, 0, -1), Fz = |phi_1|^2 - |phi_-1|^2
-    const DF ar = dw_add(dw_add(dw_mul(fx[1], fx[0]), dw_mul(fy[1], fy[0])),
-                         dw_add(dw_mul(fx[2], fx[1]), dw_mul(fy[2], fy[1])));
-    const DF ai = dw_add(dw_sub(dw_mul(fx[1], fy[0]), dw_mul(fy[1], fx[0])),
-                         dw_sub(dw_mul(fx[2], fy[1]), dw_mul(fy[2], fx[1])));
-    const DF Fz = dw_sub(m[0], m[2]);
-    DF fr[3], fi[3];
-    fr[0] = dw_add(dw_mul(Fz, fx[0]), dw_sub(dw_mul(ar, fx[1]), dw_mul(ai, fy[1])));
-    fi[0] = dw_add(dw_mul(Fz, fy[0]), dw_add(dw_mul(ar, fy[1]), dw_mul(ai, fx[1])));
-    fr[1] = dw_add(dw_add(dw_mul(ar, fx[0]), dw_mul(ai, fy[0])), dw_sub(dw_mul(ar, fx[2]), dw_mul(ai, fy[2])));
-    fi[1] = dw_add(dw_sub(dw_mul(ar, fy[0]), dw_mul(ai, fx[0])), dw_add(dw_mul(ar, fy[2]), dw_mul(ai, fx[2])));
-    fr[2] = dw_sub(dw_add(dw_mul(ar, fx[1]), dw_mul(ai, fy[1])), dw_mul(Fz, fx[2]));
-    fi[2] = dw_sub(dw_sub(dw_mul(ar, fy[1]), dw_mul(ai, fx[1])), dw_mul(Fz, fy[2]));
-    const DF c0r = dw_mul(c0, rho);
+    DF ar = dwa_of_mul(fx[1], fx[0]), ai = dwa_of_mul(fx[1], fy[0]);
+    dwa_mul(ar, fy[1], fy[0]);
+    dwa_mul(ar, fx[2], fx[1]);
+    dwa_mul(ar, fy[2], fy[1]);
+    dwa_sub(ai, fy[1], fx[0]);
+    dwa_mul(ai, fx[2], fy[1]);
+    dwa_sub(ai, fy[2], fx[1]);
+    ar = dwa_value(ar);
+    ai = dwa_value(ai);
+    DF Fz = m[0];
+    dwa_add(Fz, -m[2].hi, -m[2].lo);
+    Fz = dwa_value(Fz);
+    const DF c0r = dw_mul(c0, rho), cz = dw_mul(c1, Fz), cr = dw_mul(c1, ar), ci = dw_mul(c1, ai);
+    // each component of H in one sum; rounded to FP64 from there
+    DF h[6];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const DF hr = dw_add(dw_add(hx[c], dw_mul(c0r, fx[c])), dw_mul(c1, fr[c]));
-      const DF hi = dw_add(dw_add(hy[c], dw_mul(c0r, fy[c])), dw_mul(c1, fi[c]));
-      A.hphi[sbase + c * npts + off] = make_double2(dw_to_double(hr), dw_to_double(hi));
+      h[2 * c] = dwa_of_mul(c0r, fx[c]);
+      h[2 * c + 1] = dwa_of_mul(c0r, fy[c]);
     }
-    acc[1] = dw_add(acc[1], dw_mul(rho, rho));
-    const DF a2 = dw_add(dw_mul(ar, ar), dw_mul(ai, ai));
-    acc[2] = dw_add(acc[2], dw_add(dw_add(a2, a2), dw_mul(Fz, Fz)));
+    dwa_mul(h[0], cz, fx[0]); dwa_mul(h[0], cr, fx[1]); dwa_sub(h[0], ci, fy[1]);
+    dwa_mul(h[1], cz, fy[0]); dwa_mul(h[1], cr, fy[1]); dwa_mul(h[1], ci, fx[1]);
+    dwa_mul(h[2], cr, fx[0]); dwa_mul(h[2], ci, fy[0]); dwa_mul(h[2], cr, fx[2]); dwa_sub(h[2], ci, fy[2]);
+    dwa_mul(h[3], cr, fy[0]); dwa_sub(h[3], ci, fx[0]); dwa_mul(h[3], cr, fy[2]); dwa_mul(h[3], ci, fx[2]);
+    dwa_mul(h[4], cr, fx[1]); dwa_mul(h[4], ci, fy[1]); dwa_sub(h[4], cz, fx[2]);
+    dwa_mul(h[5], cr, fy[1]); dwa_sub(h[5], ci, fx[1]); dwa_sub(h[5], cz, fy[2]);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) acc[3 + c] = dw_add(acc[3 + c], m[c]);
-    const long long row = off / nx;
-    const float V = trap_value<float>(A.trap, A.g, (int)(off - row * nx), (int)(row % ny), (int)(row / ny), off);
+    for (int c = 0; c < 3; ++c) {
+      dwa_add(h[2 * c], hx[c].hi, hx[c].lo);
+      dwa_add(h[2 * c + 1], hy[c].hi, hy[c].lo);
+      A.hphi[at + c * npts] = make_double2(dw_to_double(h[2 * c]), dw_to_double(h[2 * c + 1]));
+    }
+    dwa_sqd(acc[1], rho);
+    dwa_mul(acc[2], DF{ar.hi + ar.hi, ar.lo + ar.lo}, ar);
+    dwa_mul(acc[2], DF{ai.hi + ai.hi, ai.lo + ai.lo}, ai);
+    dwa_sqd(acc[2], Fz);
+    const int row = (int)(off >> Lx);
+    const float V = trap_value<float>(A.trap, A.g, (int)off & (nx - 1), row & (ny - 1), row >> Ly, off);
     const float rf = mf[0] + mf[1] + mf[2];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -260,14 +287,14 @@ __global__ void __launch_bounds__(kHyThreads, kHyBlocksPerSM) k_hy_upd(HyArgs A)
     }
   }
   double* P = A.part + (long long)s * NSLOT * A.pmax + rb;
-  if (upd) {
+  if (dphi) {
     const double v = block_max((double)dmax, scratch);
     if (threadIdx.x == 0) put_partial(P + (long long)SL_DPHIINF * A.pmax, v, true, true);
   }
   if (!red) return;
   DF all[12];
 #pragma unroll
-  for (int k = 0; k < 6; ++k) { all[k] = acc[k]; all[6 + k] = DF{acc32[k], 0.0f}; }
+  for (int k = 0; k < 6; ++k) { all[k] = dwa_value(acc[k]); all[6 + k] = DF{acc32[k], 0.0f}; }
   double v[12];
   block_reduce_dw<12>(all, v, scratch);
   const int slots[12] = {SL_Q, SL_RHO2, SL_F2, SL_M0, SL_M1, SL_M2, SL_V0, SL_V1, SL_V2, SL_C0, SL_C1, SL_C2};
