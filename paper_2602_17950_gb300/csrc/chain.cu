@@ -52,13 +52,13 @@ __device__ __forceinline__ void load_tw(cx_t<T>* s_tw, const cx_t<T>* tw, int n,
 // (FP32 column passes only: the code path sets the register allocation of the whole kernel).
 // FP64 tiles of 2 elements per thread transform with half their threads.
 template <class C, bool R16 = false>
-__device__ __forceinline__ void fft_lines(int off, int nlines, int NP, int L, int ept) {
+__device__ __forceinline__ void fft_lines(int off, int nlines, int NP, int L, int ept, int down = 0) {
   if constexpr (R16 && sizeof(C) == 8) {
-    if (ept == 16) { fft_lines_e<C, 16>(off, nlines, NP, L); return; }
+    if (ept == 16) { fft_lines_e<C, 16>(off, nlines, NP, L, down); return; }
   }
-  if (ept == 8) fft_lines_e<C, 8>(off, nlines, NP, L);
-  else if (ept == 4 || sizeof(C) == 16) fft_lines_e<C, 4>(off, nlines, NP, L);
-  else if constexpr (sizeof(C) == 8) fft_lines_e<C, 2>(off, nlines, NP, L);
+  if (ept == 8) fft_lines_e<C, 8>(off, nlines, NP, L, down);
+  else if (ept == 4 || sizeof(C) == 16) fft_lines_e<C, 4>(off, nlines, NP, L, down);
+  else if constexpr (sizeof(C) == 8) fft_lines_e<C, 2>(off, nlines, NP, L, down);
 }
 
 // padded length of a column line in shared memory
@@ -314,9 +314,10 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
   // forward transforms of both arrays' lines; the inverse ones are their values at index -j
   copy_wait();
   __syncthreads();
-  fft_lines<C>(b0, two ? 6 * R : 3 * R, NP, Lx, ept);
-
-  const W inv_n = (W)1 / (W)npts;
+  // the 1/npts of the whole inverse transform: FP64 transforms scale their results by powers of two for nothing
+  const int Ln = Lx + Ly + A.g.log2n[2];
+  fft_lines<C>(b0, two ? 6 * R : 3 * R, NP, Lx, ept, MODE == ROW_INV_PLAIN ? 0 : Ln);
+  const W inv_n = sizeof(T) == 4 ? (W)1 / (W)npts : (W)1;
   if (MODE == ROW_INV_PLAIN) {
     const W sc = (W)A.scale;
     for (int e = threadIdx.x; e < per; e += blockDim.x) {
@@ -457,15 +458,16 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
           dwa_sq(pp, u[c].y);
         }
       }
-      W hpp = (W)0, hphip = (W)0, Rv = (W)0, rf = (W)0, rp = (W)0;
+      W mx_[3], mf[3], mp[3];   // Re(f conj(u)), |f|^2, |u|^2 per component
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        hpp += lin_r[c] * u[c].x + lin_i[c] * u[c].y;
-        hphip += h[c].x * u[c].x + h[c].y * u[c].y;
-        Rv += f[c].x * u[c].x + f[c].y * u[c].y;
-        rf += f[c].x * f[c].x + f[c].y * f[c].y;
-        rp += u[c].x * u[c].x + u[c].y * u[c].y;
+        acc[0] += lin_r[c] * u[c].x + lin_i[c] * u[c].y;
+        acc[1] += h[c].x * u[c].x + h[c].y * u[c].y;
+        mx_[c] = f[c].x * u[c].x + f[c].y * u[c].y;
+        mf[c] = f[c].x * f[c].x + f[c].y * f[c].y;
+        mp[c] = u[c].x * u[c].x + u[c].y * u[c].y;
       }
+      const W Rv = mx_[0] + mx_[1] + mx_[2], rf = mf[0] + mf[1] + mf[2], rp = mp[0] + mp[1] + mp[2];
       // spin vectors F(Phi), F(P) and the symmetric cross term Re F~(Phi, P), through
       // a(Phi + e P) = a(Phi) + e (a1 + a2) + e^2 a(P); Re F~ is half the e coefficient of F:
       // F_xy . G_xy = 2 Re(conj(a_F) a_G)
@@ -475,11 +477,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
       spin_a<W>(f[0], u[1], f[2], a1x, a1y);
       spin_a<W>(u[0], f[1], u[2], a2x, a2y);
       const W aXx = a1x + a2x, aXy = a1y + a2y;    // twice the cross term's a
-      const W FFz = (f[0].x * f[0].x + f[0].y * f[0].y) - (f[2].x * f[2].x + f[2].y * f[2].y);
-      const W FPz = (u[0].x * u[0].x + u[0].y * u[0].y) - (u[2].x * u[2].x + u[2].y * u[2].y);
-      const W FXz = (f[0].x * u[0].x + f[0].y * u[0].y) - (f[2].x * u[2].x + f[2].y * u[2].y);
-      acc[0] += hpp;
-      acc[1] += hphip;
+      const W FFz = mf[0] - mf[2], FPz = mp[0] - mp[2], FXz = mx_[0] - mx_[2];
       if (MODE == ROW_INV_P) accR += Rv;
       acc[2] += rf * Rv;
       acc[3] += rf * rp;
@@ -541,8 +539,11 @@ __global__ void __launch_bounds__(kThreads, row_blocks<T, MODE>()) k_row(ChainAr
 // col_line_len, so the transforms run exactly as in the row passes and the
 // transposing accesses (consecutive threads on consecutive columns) fall on
 // distinct banks.
+// whether a pass has a second tile of three components
+constexpr bool col_two(int mode) { return mode == COL_YMID_H || mode == COL_YINV_H; }
+
 template <class T, int MODE>
-__global__ void __launch_bounds__(kThreads) k_col(ChainArgs<T> A, int axis, int TC, int ept) {
+__global__ void __launch_bounds__(kThreads, 2) k_col(ChainArgs<T> A, int axis, int TC, int ept) {
   using C = cx_t<T>;
   using W = T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -564,7 +565,7 @@ __global__ void __launch_bounds__(kThreads) k_col(ChainArgs<T> A, int axis, int 
   const int NPL = col_line_len<C>(na, TC);        // padded line length
   const int CS = TC * NPL;                     // component stride in smem
   C* buf2 = buf + 3 * CS;            // second 3-component tile (YMID_H, YINV_H)
-  double* red = (double*)(buf2 + 3 * CS);
+  double* red = (double*)(col_two(MODE) ? buf2 + 3 * CS : buf2);
   const SolveState& S = A.st[s];
   const PhysDev& ph = A.phys[s];
   const W piA = geo_piL<W>(A.g, axis);
@@ -600,7 +601,10 @@ __global__ void __launch_bounds__(kThreads) k_col(ChainArgs<T> A, int axis, int 
   copy_wait();
   __syncthreads();
 
-  W acc[3] = {(W)0, (W)0, (W)0};
+  constexpr int NK = sizeof(T) == 4 ? 9 : 3;
+  W acc[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) acc[k] = (W)0;
   // one transform, or (the middle passes) a forward one, the work in k and the inverse one: a loop
   // around one inlined copy of the transforms.  The inverse transforms are forward ones whose values
   // are read at index -j
@@ -616,47 +620,28 @@ __global__ void __launch_bounds__(kThreads) k_col(ChainArgs<T> A, int axis, int 
       }
       __syncthreads();
     } else if (phase == 1) {
-      if (sizeof(T) == 4 && (MODE == COL_YMID_H || MODE == COL_MID_H) && A.xhat) {
-        // GPSOC_HYBRID P chain: buf holds the full spectrum of P.  Advance the stored spectrum
-        // of Phi by the step applied this iteration (Phi_hat <- g (c Phi_hat + t P_hat_prev)),
-        // keep this P_hat, and sum 1/2 |k|^2 |Phi_hat_l|^2 and 1/2 |k|^2 Re(Phi_hat_l conj P_hat_l)
-        const bool upd = A.khat_upd && S.upd_applied;
-        const W usc = pick<W>(S.upd_scale, S.fupd_scale);
-        const W uc = usc * pick<W>(S.upd_c, S.fupd_c), us = usc * pick<W>(S.upd_s, S.fupd_s);
-        W kacc[6] = {(W)0, (W)0, (W)0, (W)0, (W)0, (W)0};
-        for (int j = j0; j < na; j += dj) {
-          const W ka = wavenum<W>(j, na, piA);
-          const W k2h = k2c + (W)0.5 * ka * ka;
-          const long long at = col + ((long long)j << Li);
-          C xv[3], po[3];
+      // pointwise in k: the kinetic + SOC symbol (H chains) or the kinetic preconditioner; with
+      // YMID_H also G_c = F_y^-1[v_y F_y A_c] in buf2
+      const bool use_pd = (A.sc.opts.precond == GPSOC_PRECOND_COMBINED || A.sc.opts.precond == GPSOC_PRECOND_KINETIC);
+      const W gx = g * kx;
+      // GPSOC_HYBRID P chain: buf holds the full spectrum of P.  Advance the stored spectrum of Phi by
+      // the step applied this iteration (Phi_hat <- g (c Phi_hat + t P_hat_prev)), keep this P_hat, and
+      // sum 1/2 |k|^2 |Phi_hat_l|^2 and 1/2 |k|^2 Re(Phi_hat_l conj P_hat_l)
+      const bool hat = sizeof(T) == 4 && (MODE == COL_YMID_H || MODE == COL_MID_H) && A.xhat;
+      const bool upd = hat && A.khat_upd && S.upd_applied;
+      const W usc = pick<W>(S.upd_scale, S.fupd_scale);
+      const W uc = usc * pick<W>(S.upd_c, S.fupd_c), us = usc * pick<W>(S.upd_s, S.fupd_s);
+      for (int j = j0; j < na; j += dj) {
+        const int i1 = sidx(0, j), i2 = sidx(1, j), i3 = sidx(2, j);
+        const long long at = col + ((long long)j << Li);
+        C xv[3], po[3];
+        if (hat) {
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
             xv[c] = A.xhat[at + c * npts];
             if (upd) po[c] = A.phat[at + c * npts];
           }
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const C pv = buf[sidx(c, j)];
-            if (upd) {
-              xv[c] = mk<C>(uc * xv[c].x + us * po[c].x, uc * xv[c].y + us * po[c].y);
-              A.xhat[at + c * npts] = xv[c];
-            }
-            A.phat[at + c * npts] = pv;
-            kacc[c] += k2h * (xv[c].x * xv[c].x + xv[c].y * xv[c].y);
-            kacc[3 + c] += k2h * (xv[c].x * pv.x + xv[c].y * pv.y);
-          }
         }
-        const bool kmx[6] = {false, false, false, false, false, false};
-        const int kslots[6] = {SL_KPHI0, SL_KPHI1, SL_KPHI2, SL_KX0, SL_KX1, SL_KX2};
-        store_partials<6, W>(kacc, kslots, kmx, red, A.part, (long long)s * NSLOT, A.pmax, tb);
-      }
-
-      // pointwise in k: the kinetic + SOC symbol (H chains) or the kinetic preconditioner; with
-      // YMID_H also G_c = F_y^-1[v_y F_y A_c] in buf2
-      const bool use_pd = (A.sc.opts.precond == GPSOC_PRECOND_COMBINED || A.sc.opts.precond == GPSOC_PRECOND_KINETIC);
-      const W gx = g * kx;
-      for (int j = j0; j < na; j += dj) {
-        const int i1 = sidx(0, j), i2 = sidx(1, j), i3 = sidx(2, j);
         const W ka = wavenum<W>(j, na, piA);
         const W k2h = k2c + (W)0.5 * ka * ka;
         if (MODE == COL_MID_PRE) {
@@ -679,6 +664,19 @@ __global__ void __launch_bounds__(kThreads) k_col(ChainArgs<T> A, int axis, int 
             buf2[i1] = cscale(p1, ka);
             buf2[i2] = cscale(p0, ka);
             buf2[i3] = cscale(pm, ka);
+          }
+          if (hat) {
+            const C pv[3] = {p1, p0, pm};
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+              if (upd) {
+                xv[c] = mk<C>(uc * xv[c].x + us * po[c].x, uc * xv[c].y + us * po[c].y);
+                A.xhat[at + c * npts] = xv[c];
+              }
+              A.phat[at + c * npts] = pv[c];
+              acc[3 + c] += k2h * (xv[c].x * xv[c].x + xv[c].y * xv[c].y);
+              acc[6 + c] += k2h * (xv[c].x * pv[c].x + xv[c].y * pv[c].y);
+            }
           }
           // kinetic per component (Parseval): sum 1/2 |k|^2 |phat_l|^2
           acc[0] += k2h * (p1.x * p1.x + p1.y * p1.y);
@@ -728,9 +726,13 @@ __global__ void __launch_bounds__(kThreads) k_col(ChainArgs<T> A, int axis, int 
     }
   }
   if (MODE == COL_MID_H || MODE == COL_YMID_H) {
-    const bool mx[3] = {false, false, false};
-    const int slots[3] = {SL_KIN0, SL_KIN1, SL_KIN2};
-    store_partials<3, W>(acc, slots, mx, red, A.part, (long long)s * NSLOT, A.pmax, tb);
+    const int slots[9] = {SL_KIN0, SL_KIN1, SL_KIN2, SL_KPHI0, SL_KPHI1, SL_KPHI2, SL_KX0, SL_KX1, SL_KX2};
+    W aa[NK];
+    int ss[NK];
+    const bool mx[NK] = {};
+#pragma unroll
+    for (int k = 0; k < NK; ++k) { aa[k] = acc[k]; ss[k] = slots[k]; }
+    store_partials<NK, W>(aa, ss, mx, red, A.part, (long long)s * NSLOT, A.pmax, tb);
   }
 }
 
@@ -921,11 +923,11 @@ static size_t row_smem(const Geo& g, int mode, int nsolve) {
 }
 
 template <class T>
-static size_t col_smem(const Geo& g, int axis, int nsolve) {
+static size_t col_smem(const Geo& g, int axis, int nsolve, int mode) {
   using C = cx_t<T>;
   const int tc = col_tc<T>(g, axis, nsolve);
   const int CS = col_line_len<C>(g.n[axis], tc) * tc;
-  return sizeof(C) * (fft_padded_len<C>(g.n[axis]) + 6 * CS) + kRedDoubles * sizeof(double);
+  return sizeof(C) * (fft_padded_len<C>(g.n[axis]) + (col_two(mode) ? 6 : 3) * CS) + kRedDoubles * sizeof(double);
 }
 
 template <class T, int MODE>
@@ -960,7 +962,7 @@ static void col_go(int axis, const ChainArgs<T>& a, cudaStream_t st) {
   int tc, ept, threads;
   col_cfg<T>(a.g, axis, a.nsolve, tc, ept, threads);
   const int nb = col_blocks_per_solve<T>(a.g, axis, a.nsolve) * a.nsolve;
-  const size_t sm = col_smem<T>(a.g, axis, a.nsolve);
+  const size_t sm = col_smem<T>(a.g, axis, a.nsolve, MODE);
   launch_pdl(k_col<T, MODE>, nb, threads, sm, st, a, axis, tc, ept);
 }
 

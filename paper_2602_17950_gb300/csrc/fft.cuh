@@ -198,7 +198,8 @@ struct FftPad16 { __device__ __forceinline__ int operator()(int e) const { retur
 
 // Forward transforms, in place, of nlines lines of padded length NP that start `off` values behind
 // the start of the dynamic shared memory, which holds the twiddle table.  Every thread of the
-// block calls it, the lines complete in shared memory; they are complete again on return.
+// block calls it, the lines complete in shared memory; they are complete again on return.  FP64 results
+// are scaled by 2^-down.
 //
 // A line belongs to N/E consecutive threads.  When these are within one warp (N/E <= 32: lines up
 // to 256 with 8 elements per thread) its passes need no block barrier, only the warp's; before,
@@ -208,7 +209,7 @@ struct FftPad16 { __device__ __forceinline__ int operator()(int e) const { retur
 // every transform of a kernel: unrolled passes are 10 to 20 KB of instructions, run once or twice by a block, and a third of
 // the stalls of the FP64 column passes was waiting for them (ncu, no_instruction) with three.
 template <class C, int E>
-__device__ __forceinline__ void fft_lines_e(int off, int nlines, int NP, int L) {
+__device__ __forceinline__ void fft_lines_e(int off, int nlines, int NP, int L, int down) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_key[32];
   const C* tw = reinterpret_cast<const C*>(smem_raw);
@@ -225,7 +226,7 @@ __device__ __forceinline__ void fft_lines_e(int off, int nlines, int NP, int L) 
     int g = g0;
     asm volatile("" : "+r"(g));   // keeps every pass's addresses from being computed ahead of the loop, into spills
     if constexpr (sizeof(C) == 16)
-      fx_fft<E>(reinterpret_cast<FxC*>(p), act, g, L, reinterpret_cast<const FxW*>(tw), s_key, warp, FftPad16{});
+      fx_fft<E>(reinterpret_cast<FxC*>(p), act, g, L, down, reinterpret_cast<const FxW*>(tw), s_key, warp, FftPad16{});
     else
       stockham_fft<C, E>(p, act, g, L, tw, warp);
   }

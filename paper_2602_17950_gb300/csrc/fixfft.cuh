@@ -17,7 +17,7 @@
 // The values of a line are complex numbers of one transform, so one exponent per line is what
 // FP64 butterflies would meet too: they add its largest value into every output.
 //
-// Lines holding an infinity or a NaN come back as NaN; values below 2^-1022 come back as zero.
+// Lines holding an infinity or a NaN come back as NaN.
 #pragma once
 
 #include <stdint.h>
@@ -118,31 +118,64 @@ GPSOC_FX int fx_clz(unsigned v) {   // v != 0
 // the upper word without its sign: its maximum over a line gives the line's exponent field
 GPSOC_FX int fx_key(double d) { return (int)((unsigned)(fx_bits(d) >> 32) & 0x7fffffffu); }
 
+// shifts of a 64-bit value held as two words, by any distance >= 0
+GPSOC_FX void fx_shr(unsigned& h, unsigned& l, int n) {
+  if (n >= 32) { l = h; h = 0; n -= 32; }
+#if defined(__CUDA_ARCH__)
+  l = __funnelshift_rc(l, h, n);
+  h = __funnelshift_rc(h, 0u, n);
+#else
+  if (n >= 32) { l = h; h = 0; if (n > 32) l = 0; return; }
+  if (n) { l = (l >> n) | (h << (32 - n)); h >>= n; }
+#endif
+}
+GPSOC_FX unsigned fx_shl(unsigned h, unsigned l, int n) {   // upper word, 0 <= n < 32
+#if defined(__CUDA_ARCH__)
+  return __funnelshift_l(l, h, n);
+#else
+  return n ? (h << n) | (l >> (32 - n)) : h;
+#endif
+}
 // d in units of 2^(em - 1022 - f): em the line's exponent field (>= 1), |result| < 2^f, f in [53, 62]
 GPSOC_FX long long fx_of(double d, int em, int f) {
   const unsigned long long b = fx_bits(d);
-  const int e = (int)(b >> 52) & 0x7ff;
-  unsigned long long m = b & 0xfffffffffffffULL;
-  if (e) m |= 0x10000000000000ULL;
-  const int sh = em - (e ? e : 1);
-  m = (sh < 64) ? (m << (f - 53)) >> sh : 0;
-  return (long long)b < 0 ? -(long long)m : (long long)m;
+  const unsigned H = (unsigned)(b >> 32), L = (unsigned)b;
+  const int e = (int)(H >> 20) & 0x7ff;
+  unsigned h = H & 0xfffffu;
+  if (e) h |= 0x100000u;
+  h = fx_shl(h, L, f - 53);
+  unsigned l = L << (f - 53);
+  fx_shr(h, l, em - (e ? e : 1));
+  const unsigned long long sg = (unsigned long long)(long long)((int)H >> 31);
+  return (long long)(((((unsigned long long)h << 32) | l) ^ sg) - sg);
 }
-// v 2^s rounded to FP64
-GPSOC_FX double fx_to(long long v, int s) {
-  const unsigned long long sign = (unsigned long long)v & 0x8000000000000000ULL;
-  unsigned long long m = (v < 0) ? 0ULL - (unsigned long long)v : (unsigned long long)v;
-  const unsigned h = (unsigned)(m >> 32);
-  const int lz = h ? fx_clz(h) : 32 + fx_clz((unsigned)m | 1u);
-  m <<= lz;
-  const int e = 1023 + 63 + s - lz;
+// The unit 2^s of a line's results: fx_to(v, 1086 + s) where s is plain; for exponents at the ends of the
+// FP64 range (or a line with an infinity or a NaN, s >= 2048) fx_to(v, 1086) and the two factors of 2^s
+struct FxUnit { double f1, f2; };
+GPSOC_FX bool fx_plain(int s) { return s > 64 - 1086 && s < 2047 - 1086; }
+GPSOC_FX double fx_pow2(int e) {
+  return e >= 1024 ? fx_double(0x7ff0000000000000ULL) : e < -1022 ? 0.0 : fx_double((unsigned long long)(e + 1023) << 52);
+}
+GPSOC_FX FxUnit fx_unit(int s) {
+  FxUnit u;
+  u.f1 = s >= 2048 ? fx_double(0x7ff8000000000000ULL) : fx_pow2(s / 2);
+  u.f2 = fx_pow2(s - s / 2);
+  return u;
+}
+// v 2^(base - 1086) rounded to FP64, 64 < base < 2047
+GPSOC_FX double fx_to(long long v, int base) {
+  const unsigned sg = (unsigned)((int)(v >> 32) >> 31);
+  const unsigned long long m = (unsigned long long)((v ^ (v >> 63)) - (v >> 63));
+  unsigned l = (unsigned)m, h = (unsigned)(m >> 32);
+  if (h == 0) { h = l; l = 0; base -= 32; }
+  const int lz = fx_clz(h | 1u);
+  const unsigned mh = fx_shl(h, l, lz), ml = l << lz;
+  const unsigned rl = fx_shl(mh, ml, 21), up = (ml >> 10) & 1u;   // bits 42..11, and the first one dropped
   // the leading one adds 1 to the exponent field, and so does a carry out of the rounding
-  unsigned long long b = ((unsigned long long)(unsigned)(e - 1) << 52) + (m >> 11) + ((m >> 10) & 1);
-  if (e <= 0 || v == 0) b = 0;
-  if (e >= 2047) b = 0x7ff0000000000000ULL;
-  return fx_double(b | sign);
+  unsigned long long b = ((((unsigned long long)((mh >> 11) + ((unsigned)(base - lz - 1) << 20))) << 32) | rl) + up;
+  if (h == 0) b = 0;
+  return fx_double(b | ((unsigned long long)(sg & 0x80000000u) << 32));
 }
-
 // ------------------------------------------------------------------ arithmetic
 // signed halves of a value: a = h 2^32 + l
 GPSOC_FX void fx_halves(long long a, int& h, int& l) {
@@ -261,10 +294,11 @@ __device__ __forceinline__ void fx_sync(bool warp) {
 
 // One pass of radix R (see stockham_pass) over the line at p: FIRST reads FP64 values and scales
 // the line, `last` writes FP64 values; between passes the line holds fixed-point values in the
-// same places.  sc: exponent of a unit of the line.
+// same places.  sc: exponent of a unit of the line; the results are scaled by 2^-down (the 1/n of
+// inverse transforms, for nothing).
 template <int R, int E, bool FIRST, class Pad>
 __device__ __forceinline__ void fx_pass(FxC* p, bool act, int g0, int N, int Ns, const FxW* tw, bool last, int& sc,
-                                        int* s_key, bool warp, Pad pad) {
+                                        int down, int* s_key, bool warp, Pad pad) {
   constexpr int PER = E / R;
   const int NR = N / R, G = N / E;
   FxC v[E];
@@ -304,7 +338,7 @@ __device__ __forceinline__ void fx_pass(FxC* p, bool act, int g0, int N, int Ns,
         v[e].x = fx_of(__longlong_as_double(v[e].x), em, F);
         v[e].y = fx_of(__longlong_as_double(v[e].y), em, F);
       }
-      sc = em == 0x7ff ? 4096 : em - 1022 - F;
+      sc = em == 0x7ff ? 4096 : em - 1022 - F - down;
     } else {
       sc += kFxShift<E>;
     }
@@ -322,13 +356,21 @@ __device__ __forceinline__ void fx_pass(FxC* p, bool act, int g0, int N, int Ns,
       fx_dft<false, R>(&v[u * R]);
       const int ob = (g - k) * R + k;
       if (last) {
+        const int base = fx_plain(sc) ? 1086 + sc : 1086;
 #pragma unroll
         for (int q = 0; q < R; ++q) {
-          // sc >= 2048: the line holds an infinity or a NaN
           FxC z = v[u * R + q];
-          z.x = sc < 2048 ? __double_as_longlong(fx_to(z.x, sc)) : 0x7ff8000000000000LL;
-          z.y = sc < 2048 ? __double_as_longlong(fx_to(z.y, sc)) : 0x7ff8000000000000LL;
+          z.x = __double_as_longlong(fx_to(z.x, base));
+          z.y = __double_as_longlong(fx_to(z.y, base));
           p[pad(ob + q * Ns)] = z;
+        }
+        if (!fx_plain(sc)) {   // rare, and not unrolled: exponents at the ends of the FP64 range, infinities, NaN
+          const FxUnit unit = fx_unit(sc);
+#pragma unroll 1
+          for (int q = 0; q < R; ++q) {
+            double2* z = reinterpret_cast<double2*>(&p[pad(ob + q * Ns)]);
+            *z = make_double2((z->x * unit.f1) * unit.f2, (z->y * unit.f1) * unit.f2);
+          }
         }
       } else {
 #pragma unroll
@@ -341,17 +383,18 @@ __device__ __forceinline__ void fx_pass(FxC* p, bool act, int g0, int N, int Ns,
 
 // The transform of length N = 2^L of one line per G = N/E threads: FP64 values in and out.
 template <int E, class Pad>
-__device__ __forceinline__ void fx_fft(FxC* p, bool act, int g0, int L, const FxW* tw, int* s_key, bool warp, Pad pad) {
+__device__ __forceinline__ void fx_fft(FxC* p, bool act, int g0, int L, int down, const FxW* tw, int* s_key, bool warp,
+                                       Pad pad) {
   const int N = 1 << L;
   constexpr int LE = (E == 8) ? 3 : 2;
   const int rem = L % LE, full = L / LE;
   int Ns = E, n = 1, sc = 0;
-  if (rem == 1) { fx_pass<2, E, true>(p, act, g0, N, 1, tw, full == 0, sc, s_key, warp, pad); Ns = 2; n = 0; }
-  else if (LE == 3 && rem == 2) { fx_pass<4, E, true>(p, act, g0, N, 1, tw, full == 0, sc, s_key, warp, pad); Ns = 4; n = 0; }
-  else fx_pass<E, E, true>(p, act, g0, N, 1, tw, full == 1, sc, s_key, warp, pad);
+  if (rem == 1) { fx_pass<2, E, true>(p, act, g0, N, 1, tw, full == 0, sc, down, s_key, warp, pad); Ns = 2; n = 0; }
+  else if (LE == 3 && rem == 2) { fx_pass<4, E, true>(p, act, g0, N, 1, tw, full == 0, sc, down, s_key, warp, pad); Ns = 4; n = 0; }
+  else fx_pass<E, E, true>(p, act, g0, N, 1, tw, full == 1, sc, down, s_key, warp, pad);
 #pragma unroll 1
   for (; n < full; ++n) {
-    fx_pass<E, E, false>(p, act, g0, N, Ns, tw, n == full - 1, sc, s_key, warp, pad);
+    fx_pass<E, E, false>(p, act, g0, N, Ns, tw, n == full - 1, sc, down, s_key, warp, pad);
     Ns *= E;
   }
 }

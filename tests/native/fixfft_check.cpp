@@ -8,6 +8,12 @@ using namespace gpsoc;
 
 static const FxTable g_table = fx_make_table();
 
+static double to(long long v, int s) {
+  if (fx_plain(s)) return fx_to(v, 1086 + s);
+  const FxUnit u = fx_unit(s);
+  return (fx_to(v, 1086) * u.f1) * u.f2;
+}
+
 template <bool INV, int R, int E>
 static void pass(const FxC* in, FxC* out, int n, int Ns, bool first) {
   const int NR = n / R, shift = kFxShift<E>;
@@ -55,8 +61,8 @@ static void line(double* d, int n) {
     sc += kFxShift<E>;
   }
   for (int i = 0; i < n; ++i) {
-    d[2 * i] = em == 0x7ff ? __builtin_nan("") : fx_to(b[i].x, sc);
-    d[2 * i + 1] = em == 0x7ff ? __builtin_nan("") : fx_to(b[i].y, sc);
+    d[2 * i] = to(b[i].x, em == 0x7ff ? 4096 : sc);
+    d[2 * i + 1] = to(b[i].y, em == 0x7ff ? 4096 : sc);
   }
   free(a);
   free(b);
@@ -71,6 +77,6 @@ void fx_line(double* d, int n, int e, int inverse) {
 // table entry k as (re, im) in units of 2^-62
 void fx_table(int k, long long* out) { out[0] = g_table.c[2 * k]; out[1] = g_table.c[2 * k + 1]; }
 // d -> fixed point at exponent field em with f bits -> FP64
-double fx_round_trip(double d, int em, int f) { return fx_to(fx_of(d, em, f), em - 1022 - f); }
-double fx_widen(long long v, int s) { return fx_to(v, s); }
+double fx_round_trip(double d, int em, int f) { return to(fx_of(d, em, f), em - 1022 - f); }
+double fx_widen(long long v, int s) { return to(v, s); }
 }
