@@ -741,7 +741,13 @@ __global__ void __launch_bounds__(kThreads, 2) k_col(ChainArgs<T> A, int axis, i
 // column tile and component) that still gives the launch at least kTargetBlocks
 // blocks over all solves, so small grids and single solves spread over the SMs
 // while large batches keep long coalesced line segments.
+//
+// FP32 differs where its sweeps did: row tiles are worth halving only below 176 blocks (16 x 64^2 hybrid:
+// 2 rows 1493 us, 4 rows 1410); column tiles keep 4 columns, the 32 bytes of a sector, however few
+// blocks that leaves (one 512^2 solve, 1 column 1944 us, 4 columns 1650; 256^2 1611 and 1493; 3 x 128^2 1546 and
+// 1389), and take 8 when 8 blocks per SM remain (64 x 256^2 24.7 ms and 23.4).
 static constexpr int kTargetBlocks = 304;   // two blocks per SM of a 152-SM GB300
+static constexpr int kTargetRows32 = 176;
 
 // Tuned tiles (gpsoc_tuning_set / gpsoc_autotune) override the rule below for one
 // grid, batch and precision; every launch and every block count of that key reads the
@@ -783,7 +789,8 @@ int row_rows_per_block(const Geo& g, int nsolve) {
   int R = 512 / nx;
   if (R < 1) R = 1;
   if (R > rows) R = rows;
-  while (R > 1 && (long long)nsolve * (rows / R) < kTargetBlocks) R >>= 1;
+  const int target = sizeof(T) == 4 ? kTargetRows32 : kTargetBlocks;
+  while (R > 1 && (long long)nsolve * (rows / R) < target) R >>= 1;
   return R;
 }
 
@@ -798,19 +805,27 @@ int col_tc(const Geo& g, int axis, int nsolve) {
   int tc = 1024 / na;
   if (tc < 1) tc = 1;
   if (tc > ni) tc = ni;
-  while (tc > 1 && (long long)nsolve * (ni / tc) * no < kTargetBlocks) tc >>= 1;
+  const long long columns = (long long)nsolve * ni * no;
+  while (tc > 1 && columns / tc < kTargetBlocks) tc >>= 1;
+  if (sizeof(T) == 4) {
+    if (tc < 4) tc = ni < 4 ? ni : 4;
+    else if (2 * tc <= ni && 2 * tc * na <= 2048 && columns / (2 * tc) >= 4 * kTargetBlocks) tc *= 2;
+  }
   return tc;
 }
 
 // elements per thread of the FFT passes: 16 (radix-16 passes, FP32 column passes) or 8,
 // unless the tile would then have fewer than 128 threads or a line is shorter,
 // in which case fewer (more threads, more passes); and the matching thread
-// count (multiple of 32, >= 64)
+// count (multiple of 32, >= 64).  Rows: where the blocks fill the SMs, 8 (FP32: 16 x 64^2 hybrid
+// 1493 us with 2, 1386 with 8) or at least 4 (FP64: 16 x 64^2 3118 us with 2, 3013 with 4) whatever the threads.
 template <class T>
-static int pick_ept(int work /* complex elements of the three components */, int n /* line length */,
-                    bool r16 = true) {
-  int e = (sizeof(T) == 4 && r16) ? 16 : 8;
-  while (e > 2 && (work / e < 128 || e > n)) e >>= 1;
+static int pick_ept(int work /* complex elements of the three components */, int n /* line length */, bool column,
+                    long long blocks) {
+  int e = (sizeof(T) == 4 && column) ? 16 : 8;
+  const bool full = !column && blocks >= kTargetBlocks;
+  const int least = full ? (sizeof(T) == 4 ? 8 : 4) : 2;
+  while (e > 2 && ((work / e < 128 && e > least) || e > n)) e >>= 1;
   return e;
 }
 static int round_threads(int t) {
@@ -823,7 +838,8 @@ static int row_ept(const Geo& g, int nsolve) {
   int tl, te;
   tuned<T>(g, 0, nsolve, tl, te);
   if (tl > 0 && te > 0) return te;
-  return pick_ept<T>(3 * row_rows_per_block<T>(g, nsolve) * g.n[0], g.n[0], false);
+  const int R = row_rows_per_block<T>(g, nsolve);
+  return pick_ept<T>(3 * R * g.n[0], g.n[0], false, (long long)nsolve * (g.npts / g.n[0]) / R);
 }
 
 template <class T>
@@ -832,7 +848,7 @@ static void col_cfg(const Geo& g, int axis, int nsolve, int& tc, int& ept, int& 
   const int work = 3 * tc * g.n[axis];
   int tl, te;
   tuned<T>(g, axis, nsolve, tl, te);
-  ept = (tl > 0 && te > 0) ? te : pick_ept<T>(work, g.n[axis]);
+  ept = (tl > 0 && te > 0) ? te : pick_ept<T>(work, g.n[axis], true, 0);
   threads = round_threads(work / ept);
 }
 
