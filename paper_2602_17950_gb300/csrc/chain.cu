@@ -126,8 +126,8 @@ __device__ __forceinline__ void store_partials(const W (&acc)[K], const int (&sl
 // (per-thread partial sums in T, block and grid reductions in FP64).
 //
 // Sizes are powers of two, so indices are split by shifts (integer divisions, two of them of 64 bits
-// per point, were a third of the instructions of the FP32 passes).  The tiles of the inverse passes
-// come by asynchronous copies, which are under way while the twiddle table is set up.
+// per point, were a third of the instructions of the FP32 passes).  The twiddle table is set up before the
+// wait for the kernel before; the tiles of the inverse passes come by asynchronous copies.
 template <class T, int MODE>
 __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) {
   using C = cx_t<T>;
@@ -143,9 +143,10 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
   const int bps = (int)(npts >> Lx) / R;
   const int s = blockIdx.x / bps;
   const int rb = blockIdx.x - s * bps;
+  C* s_tw = (C*)smem_raw;
+  load_tw<T>(s_tw, A.tw[0], nx, ept);
   pdl_wait();
   if (s >= A.nsolve || !gate_ok(A.st, A.gate, s)) return;
-  C* s_tw = (C*)smem_raw;
   const int b0 = fft_padded_len<C>(nx);   // the lines lie behind the table
   C* buf0 = s_tw + b0;
   const int per = R << Lx;            // elements of one component in the tile
@@ -172,7 +173,6 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
       }
     }
   }
-  load_tw<T>(s_tw, A.tw[0], nx, ept);
   // the solve's scalars, read before the transforms
   const W c0 = pick<W>(ph.c0, ph.fc0), c1 = pick<W>(ph.c1, ph.fc1), Om = pick<W>(ph.Omega, ph.fOmega);
   const W al[3] = {pick<W>(S.alpha[0], S.falpha[0]), pick<W>(S.alpha[1], S.falpha[1]), pick<W>(S.alpha[2], S.falpha[2])};
@@ -555,9 +555,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_col(ChainArgs<T> A, int axis, i
   const int bps = (int)(npts >> (La + LT));
   const int s = blockIdx.x / bps;
   const int tb = blockIdx.x - s * bps;
+  C* s_tw = (C*)smem_raw;
+  load_tw<T>(s_tw, A.tw[axis], na, ept);
   pdl_wait();
   if (s >= A.nsolve || !gate_ok(A.st, A.gate, s)) return;
-  C* s_tw = (C*)smem_raw;
   const int o = tb >> Lt;
   const int i0 = (tb - (o << Lt)) << LT;
   const int b0 = fft_padded_len<C>(na);   // the lines lie behind the table
@@ -577,8 +578,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_col(ChainArgs<T> A, int axis, i
   const int lt = t * NPL;
   auto sidx = [&](int c, int j) { return c * CS + lt + fft_pad<C>(j); };
 
-  // the in0 tile (and in1 for YINV_H) in natural order, by asynchronous copies that are under way
-  // while the twiddle table is set up
+  // the in0 tile (and in1 for YINV_H) in natural order, by asynchronous copies
   for (int j = j0; j < na; j += dj) {
     const long long at = col + ((long long)j << Li);
 #pragma unroll
@@ -587,7 +587,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_col(ChainArgs<T> A, int axis, i
       if (MODE == COL_YINV_H) copy_async(&buf2[sidx(c, j)], A.in1 + at + c * npts);
     }
   }
-  load_tw<T>(s_tw, A.tw[axis], na, ept);
   // wavenumbers of the column's inner index (the inputs are spectral along the faster axes)
   W kx, kyc;
   {

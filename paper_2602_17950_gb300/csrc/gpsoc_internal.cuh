@@ -12,7 +12,6 @@
 
 #include <cuda_runtime.h>
 #include <stdint.h>
-#include <stdlib.h>
 
 #include "../../include/gpsoc.h"
 #include "dword.cuh"
@@ -199,29 +198,14 @@ struct ChainArgs {
   int khat_upd;
 };
 
-// Programmatic dependent launch.  The iteration's kernels are launched with programmatic
-// stream serialisation (launch_pdl).  pdl_wait() waits until the kernel before it in the
-// stream has completed and its writes are visible (griddepcontrol.wait); every read of
-// data another kernel writes comes after it, only constant tables are read before.
-// pdl_trigger() (griddepcontrol.launch_dependents) lets the next kernel's blocks be
-// scheduled once every block has issued it or exited.  The passes with a fused scalar
-// tail issue it when a block has written its partial sums (last_block), so the next
-// kernel's blocks are placed on SMs this pass has left, and wait there while the last
-// block runs the tail; the others trigger at exit.  Without the launch attribute (the
-// default) the wait returns at once.
+// Programmatic dependent launch.  The kernels are launched with programmatic stream serialisation
+// (launch_pdl): once every block of a kernel has exited, the blocks of the next one are placed before
+// the kernel counts as complete and its writes are visible.  They set up what no kernel writes
+// (twiddles) and stop at pdl_wait() (griddepcontrol.wait) until then; every read of data another
+// kernel writes comes after it.  12 us of the 83 us H(Phi) of 64^2, 5 us of the 75 us of a 128^2
+// hybrid iteration.  Triggering the next kernel earlier (griddepcontrol.launch_dependents after a
+// block's own wait) placed its blocks around the running ones, on fewer SMs: 256^2 hybrid 1422 -> 1743 us.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
-// launch with programmatic stream serialisation when GPSOC_PDL=1 is set in the environment
-// (kernels that call pdl_wait before reading what earlier kernels wrote); by default the
-// kernels run in plain stream order, which measured faster for this iteration's kernels
-inline bool pdl_enabled() {
-  static const bool on = [] {
-    const char* e = getenv("GPSOC_PDL");
-    return e && e[0] == '1';
-  }();
-  return on;
-}
 
 template <class... KArgs, class... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
@@ -235,7 +219,7 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = pdl_enabled() ? 1 : 0;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args&&>(args)...);
 }
 
@@ -251,7 +235,6 @@ __device__ __forceinline__ bool gate_ok(const SolveState* st, int gate, int s) {
 // One thread's acquire-release addition orders the whole block's writes before it (they precede the
 // barrier) and the block's reads after it.
 __device__ __forceinline__ bool last_block(unsigned* cnt, int s, int bps, int* flag_smem) {
-  pdl_trigger();
   __syncthreads();
   if (threadIdx.x == 0) {
     unsigned prev;

@@ -430,15 +430,14 @@ void launch_hy_upd(const HyArgs& a, cudaStream_t st) {
   launch_pdl(k_hy_upd, a.bps * a.nsolve, kHyThreads, 0, st, a);
 }
 
-// The pass is FP64-bound: its time is that of the busiest SM.  Two 256-thread blocks
-// are resident per SM, so the grid is a whole number of waves of 2 nsm blocks (split
-// over the solves, rounded up), with about four points per thread at most.
+// Its time is that of the busiest SM.  Two 256-thread blocks are resident per SM, so the grid is a whole number of waves of 2 nsm blocks (split
+// over the solves, rounded up), with about four points per thread at most, and at least one.
 int hy_blocks_per_solve(const Geo& g, int nsolve, int nsm) {
   const long long wave = (long long)kHyBlocksPerSM * std::max(nsm, 1);
   const long long work = (long long)std::max(nsolve, 1) * g.npts;
   const long long waves = std::max(1LL, (work + wave * kHyThreads * 4 - 1) / (wave * kHyThreads * 4));
   const long long b = (wave * waves + nsolve - 1) / std::max(nsolve, 1);
-  return (int)std::max(1LL, std::min(b, g.npts));
+  return (int)std::max(1LL, std::min(b, (g.npts + kHyThreads - 1) / kHyThreads));
 }
 
 template <class T>
