@@ -8,6 +8,7 @@
 // only every `check_every` iterations.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -1724,6 +1725,7 @@ struct Bucket {
   int stage = 2;
   OptsDev o{};
   std::vector<int64_t> slot;   // ticket per slot, -1 = free
+  std::vector<int> fresh;      // slots loaded and not yet initialised
   size_t bytes = 0;
   cudaEvent_t done = nullptr;  // recorded after the last launched round of iterations
   bool in_flight = false;
@@ -1781,33 +1783,57 @@ size_t bucket_bytes(const gpsoc_grid& g, int slots, int stage) {
   return b + (4u << 20);
 }
 
+// Slot s of the bucket is for request r: its wave function goes there; init_slots makes it a running solve.
 gpsoc_status load_slot(Bucket* b, int s, const ServerReq& r) {
   gpsoc_problem* p = b->p;
   const Geo g = make_geo(p, 0);
-  const size_t off = (size_t)s * 3 * g.npts;
-  CK(cudaMemcpyAsync(p->b64.Phi + off, r.psi.data(), sizeof(double2) * 3 * g.npts, cudaMemcpyHostToDevice, p->stream));
-  const PhysDev ph = make_phys(r.par.Omega, r.par.gamma, r.par.beta0, r.par.beta1);
-  CK(cudaMemcpyAsync(p->d_phys + s, &ph, sizeof(PhysDev), cudaMemcpyHostToDevice, p->stream));
-  ElemArgs<double> e = elem_args<double>(p, g, GATE_ALL);
-  e.only = s;
-  e.in0 = p->b64.Phi;
-  EL<double>(p, EL_MASS, e);
-  ScalarArgs x = scalar_args(p, 0, PH_NORM, g);
-  x.only = s;
-  SL(p, x);
-  e.out0 = p->b64.Phi;
-  EL<double>(p, EL_SCALE, e);
-  ScalarArgs in = scalar_args(p, 0, PH_INIT, g);
-  in.only = s;
-  in.flags = 1;
-  SL(p, in);
+  CK(cudaMemcpyAsync(p->b64.Phi + (size_t)s * 3 * g.npts, r.psi.data(), sizeof(double2) * 3 * g.npts, cudaMemcpyHostToDevice,
+                     p->stream));
+  p->params[s] = r.par;
+  b->fresh.push_back(s);
+  return GPSOC_OK;
+}
+
+// The slots loaded since the last call: parameters, normalisation and PCG state (first = 1 restarts
+// beta), all of them in one set of launches (12 requests of 64^2, submission to last answer: 2210 us with a
+// set for each, 2139 with one).
+gpsoc_status init_slots(Bucket* b) {
+  gpsoc_problem* p = b->p;
+  const Geo g = make_geo(p, 0);
+  std::vector<PhysDev> ph(p->batch);   // running slots keep the values they have
+  for (int k = 0; k < p->batch; ++k)
+    ph[k] = make_phys(p->params[k].Omega, p->params[k].gamma, p->params[k].beta0, p->params[k].beta1);
+  CK(cudaMemcpyAsync(p->d_phys, ph.data(), sizeof(PhysDev) * p->batch, cudaMemcpyHostToDevice, p->stream));
+  std::sort(b->fresh.begin(), b->fresh.end());
+  for (size_t i = 0; i < b->fresh.size();) {
+    SlotMask m;
+    m.first = b->fresh[i];
+    for (; i < b->fresh.size() && b->fresh[i] < m.first + 64; ++i) {
+      m.bits |= 1ull << (b->fresh[i] - m.first);
+    }
+    ElemArgs<double> e = elem_args<double>(p, g, GATE_ALL);
+    e.only = m;
+    e.in0 = p->b64.Phi;
+    EL<double>(p, EL_MASS, e);
+    ScalarArgs x = scalar_args(p, 0, PH_NORM, g);
+    x.only = m;
+    SL(p, x);
+    e.out0 = p->b64.Phi;
+    EL<double>(p, EL_SCALE, e);
+    ScalarArgs in = scalar_args(p, 0, PH_INIT, g);
+    in.only = m;
+    in.flags = 1;
+    SL(p, in);
+  }
   if (b->fp32_phase) {
-    launch_convert<float>(p->b64.Phi + off, 0, p->b32.Phi + off, (long long)3 * g.npts, p->stream);
-    mark(p, "convert");
+    for (int s : b->fresh) {
+      const size_t off = (size_t)s * 3 * g.npts;
+      launch_convert<float>(p->b64.Phi + off, 0, p->b32.Phi + off, (long long)3 * g.npts, p->stream);
+      mark(p, "convert");
+    }
   }
   CK(cudaGetLastError());
-  // the PCG state of this slot is per solve (first = 1 restarts beta); host parameters follow
-  p->params[s] = r.par;
+  b->fresh.clear();
   return GPSOC_OK;
 }
 
@@ -2030,15 +2056,21 @@ gpsoc_status server_step_impl(gpsoc_server* s, int* busy, bool bounded, Clock::t
   for (uint64_t t : s->queue) {
     ServerReq* r = s->reqs[t];
     Bucket* b = find_or_make_bucket(s, *r, r->stage, &err);
-    if (err != GPSOC_OK) return err;
+    if (err != GPSOC_OK) break;
     if (!b) { waiting.push_back(t); continue; }
     int slot = -1;
     for (size_t k = 0; k < b->slot.size(); ++k)
       if (b->slot[k] < 0) { slot = (int)k; break; }
-    gpsoc_status st = load_slot(b, slot, *r);
-    if (st != GPSOC_OK) return st;
+    err = load_slot(b, slot, *r);
+    if (err != GPSOC_OK) break;
     b->slot[slot] = (int64_t)t;
   }
+  for (Bucket* b : s->buckets) {     // also those loaded before an error
+    if (b->fresh.empty()) continue;
+    const gpsoc_status st = init_slots(b);
+    if (err == GPSOC_OK) err = st;
+  }
+  if (err != GPSOC_OK) return err;
   s->queue.swap(waiting);
   // 3. every idle bucket that holds work starts its next round on its own stream
   const int iters = s->opts.iters_per_step > 0 ? s->opts.iters_per_step : 32;

@@ -14,6 +14,15 @@ enum Phase {
   PH_KIN            // per-component kinetic sums of the last column pass into the state (GPSOC_HYBRID)
 };
 
+// A set of solves passed to a kernel by value: every solve, or up to 64 of them from `first` on.
+struct SlotMask {
+  int first = -1;               // -1: every solve
+  unsigned long long bits = 0;
+  __host__ __device__ bool has(int s) const {
+    return first < 0 || (s >= first && s < first + 64 && ((bits >> (s - first)) & 1));
+  }
+};
+
 struct ScalarArgs {
   SolveState* st;
   const PhysDev* phys;
@@ -29,7 +38,7 @@ struct ScalarArgs {
   double* norm_scale;
   int force;          // process every solve regardless of its active flag
   const double* thetas; int n_theta; double* model_out;
-  int only = -1;      // >= 0: act on this solve only (per-slot operations of the server)
+  SlotMask only;      // solves to act on (slots the server fills)
   double inv_npts = 0.0;   // 1 / npts
   int part_dw = 0;    // the sum partials it reads are double words (FP32 passes wrote them)
 };
@@ -48,7 +57,7 @@ struct ElemArgs {
   int bps;            // blocks per solve (divides npts)
   int nsolve;
   int gate;
-  int only = -1;      // >= 0: act on this solve only (per-slot operations of the server)
+  SlotMask only;      // solves to act on (slots the server fills)
 };
 
 // GPSOC_HYBRID: the pass that opens an iteration (FP64 state, double-word arithmetic).

@@ -26,7 +26,7 @@ __global__ void k_scalar(ScalarArgs A) {
   if (s >= A.nsolve) return;
   SolveState& S = A.st[s];
   const int ph_ = A.phase;
-  if (A.only >= 0 && s != A.only) return;
+  if (!A.only.has(s)) return;
   if (ph_ != PH_INIT && ph_ != PH_NORM && !A.force && !S.active) return;
   ScalarCtx X{A.st, A.phys, A.part, A.pmax, A.nb_row, A.nb_col, A.npts, A.dV, A.opts, A.flags, A.inv_npts, A.part_dw};
   switch (ph_) {
@@ -87,7 +87,7 @@ __global__ void k_elem(ElemArgs<T> A) {
   const int s = blockIdx.x / bps, rb = blockIdx.x % bps;
   if (s >= A.nsolve) return;
   const SolveState& S = A.st[s];
-  if (A.only >= 0 && s != A.only) return;
+  if (!A.only.has(s)) return;
   if (!gate_ok(A.st, A.gate, s)) return;
   const long long npts = A.npts;
   const long long per = npts / bps;
