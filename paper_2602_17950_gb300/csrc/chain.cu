@@ -105,7 +105,8 @@ __device__ __forceinline__ double max_pos(double a, double b) {
 // (FP32 partials are added in double-float, which carries more bits than the partials hold)
 template <int K, class W>
 __device__ __forceinline__ void store_partials(const W (&acc)[K], const int (&slots)[K], const bool (&mx)[K],
-                                               double* red, double* part, long long sbase_slot, int pmax, int blk) {
+                                               double* red, double* part, long long sbase_slot, int pmax, int blk, int nb,
+                                               unsigned* gcnt, double* tail) {
   double v[K];
   if constexpr (sizeof(W) == 4 && K >= 2) {
     block_reduce_df<K>(acc, v, red);     // FP32 partials: double-float sums on the FP32 pipes
@@ -119,6 +120,9 @@ __device__ __forceinline__ void store_partials(const W (&acc)[K], const int (&sl
     block_reduce<K>(v, red, mx);
   }
   put_partials<K>(part, sbase_slot, pmax, blk, slots, v, mx, sizeof(W) == 4);
+  using V = std::conditional_t<sizeof(W) == 4, DF, double>;
+  if (K == 1 && mx[0]) group_max<V>(part + sbase_slot * pmax, pmax, slots[0], blk, nb, gcnt, tail);
+  else group_sums<V, K>(part + sbase_slot * pmax, pmax, slots, blk, nb, gcnt, tail);
 }
 
 // ============================================================== row passes (x axis)
@@ -156,6 +160,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
   // scratch of a fused scalar step: over the tile, which is done with by then (32 doubles per warp are
   // at most half of its 24 or 48 bytes per element)
   double* tail = (double*)smem_raw;
+  unsigned* gcnt = A.gcnt + (long long)s * A.gmax;
   // this tile's first point; component c is npts further on
   const long long base = (long long)s * 3 * npts + ((long long)rb * R << Lx);
   const int row0 = rb * R;
@@ -303,7 +308,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
       const bool mx[1] = {MODE != ROW_FWD_PROJ};
       const int slots[1] = {(MODE == ROW_FWD_PROJ) ? (int)SL_P2
                             : (MODE == ROW_FWD_PRE || MODE == ROW_FWD_PRE_HY) ? (int)SL_RINF : (int)SL_DPHIINF};
-      store_partials<1, W>(acc, slots, mx, red, A.part, sslot, A.pmax, rb);
+      store_partials<1, W>(acc, slots, mx, red, A.part, sslot, A.pmax, rb, bps, gcnt, tail);
     }
     if ((MODE == ROW_FWD_PRE || MODE == ROW_FWD_PRE_HY) && A.fuse && last_block(A.cnt, s, bps, &last_flag))
       sc_res(A.sc, s, tail);
@@ -372,7 +377,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
     }
     const bool mx[5] = {false, false, false, false, false};
     const int slots[5] = {SL_RZ, SL_RPZ, SL_ZPHI, SL_PPHI, SL_RP};
-    store_partials<5, W>(acc, slots, mx, red, A.part, sslot, A.pmax, rb);
+    store_partials<5, W>(acc, slots, mx, red, A.part, sslot, A.pmax, rb, bps, gcnt, tail);
     if (A.fuse && last_block(A.cnt, s, bps, &last_flag)) sc_beta<PV>(A.sc, s, tail);
     return;
   }
@@ -391,7 +396,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
     const int row = row0 + r;
     C u[3];  // Phi for ROW_INV_H, P for ROW_INV_P / ROW_INV_LIN
     C f[3], h[3];
-    double2 g64[3];
+    C fl[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       u[c] = __ldg(A.in2 + at + c * npts);
@@ -399,7 +404,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
         f[c] = __ldg(A.in3 + at + c * npts);
         h[c] = __ldg(A.in4 + at + c * npts);
       }
-      if (MODE == ROW_INV_P_HY) g64[c] = __ldg(A.phi64 + at + c * npts);
+      if (MODE == ROW_INV_P_HY) fl[c] = __ldg(A.philo + at + c * npts);
     }
     const W ox = Omn * coord<W>(A.g, 0, j);
     const W V = trap_value<W>(A.trap, A.g, j, row & (ny - 1), row >> Ly, at - (long long)s * 3 * npts);
@@ -447,13 +452,13 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
     } else {  // ROW_INV_P: step-model reductions (Eqs. an, bn and the sin/cos form of E(theta))
       if constexpr (MODE == ROW_INV_P_HY) {
         // H_lin P kept for the update of H_lin Phi by linearity; the radial part of P (P's FP32
-        // values against the FP64 Phi) and ||P||^2 to double-word accuracy for the exact tangent
+        // values against Phi's double words, as the opening pass left them) and ||P||^2 to double-word accuracy for the exact tangent
         // correction and the normalisation of the step
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           A.out0[at + c * npts] = mk<C>(lin_r[c], lin_i[c]);
-          dwa_mulf(rphi, dw_of(g64[c].x), u[c].x);
-          dwa_mulf(rphi, dw_of(g64[c].y), u[c].y);
+          dwa_mulf(rphi, DF{f[c].x, fl[c].x}, u[c].x);
+          dwa_mulf(rphi, DF{f[c].y, fl[c].y}, u[c].y);
           dwa_sq(pp, u[c].x);
           dwa_sq(pp, u[c].y);
         }
@@ -496,7 +501,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
   if (MODE == ROW_INV_H) {
     const bool mx12[12] = {};
     const int slots[12] = {SL_Q, SL_RHO2, SL_F2, SL_V0, SL_V1, SL_V2, SL_C0, SL_C1, SL_C2, SL_M0, SL_M1, SL_M2};
-    store_partials<12, W>(acc, slots, mx12, red, A.part, sslot, A.pmax, rb);
+    store_partials<12, W>(acc, slots, mx12, red, A.part, sslot, A.pmax, rb, bps, gcnt, tail);
     if (A.fuse && last_block(A.cnt, s, bps, &last_flag)) sc_obs<PV>(A.sc, s, tail);
   } else {
     const int slots[14] = {SL_HPP, SL_HPHIP, SL_IFR, SL_IFP, SL_IRR, SL_IRP, SL_IPP,
@@ -510,13 +515,14 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
       double v[14];
       block_reduce_dw<14>(all, v, red);
       put_partials<14>(A.part, sslot, A.pmax, rb, slots, v, mx, true);
+      group_sums<DF, 14>(A.part + sslot * A.pmax, A.pmax, slots, rb, bps, gcnt, tail);
     } else {
       W a13[13];
       int s13[13];
       const bool m13[13] = {};
 #pragma unroll
       for (int k = 0; k < 13; ++k) { a13[k] = k < 12 ? acc[k] : accR; s13[k] = slots[k]; }
-      store_partials<13, W>(a13, s13, m13, red, A.part, sslot, A.pmax, rb);
+      store_partials<13, W>(a13, s13, m13, red, A.part, sslot, A.pmax, rb, bps, gcnt, tail);
     }
     if (A.fuse && last_block(A.cnt, s, bps, &last_flag)) sc_step<PV>(A.sc, s, tail);
   }
@@ -731,7 +737,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_col(ChainArgs<T> A, int axis, i
     const bool mx[NK] = {};
 #pragma unroll
     for (int k = 0; k < NK; ++k) { aa[k] = acc[k]; ss[k] = slots[k]; }
-    store_partials<NK, W>(aa, ss, mx, red, A.part, (long long)s * NSLOT, A.pmax, tb);
+    store_partials<NK, W>(aa, ss, mx, red, A.part, (long long)s * NSLOT, A.pmax, tb, bps,
+                          A.gcnt + (long long)s * A.gmax, (double*)smem_raw);
   }
 }
 

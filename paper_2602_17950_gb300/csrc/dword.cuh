@@ -167,7 +167,7 @@ GPSOC_DW double widen_f(float f) {
 // exact subtractions 1.m 2^q - 2^q, which normalise them.  Finite x with |x| < 2^-126
 // gives 0 (its low word vanishes below 2^-80); x beyond the FP32 range gives inf, NaN
 // stays NaN.
-GPSOC_DW DF dw_of(double x) {
+GPSOC_DW DF dw_of_any(double x) {
   const unsigned H = d_hi(x), L = d_lo(x);
   const unsigned sign = H & 0x80000000u;
   const int E = (int)((H >> 20) & 0x7ffu);                   // biased binary64 exponent
@@ -188,6 +188,20 @@ GPSOC_DW DF dw_of(double x) {
     r.hi = (E == 2047 && ((H & 0xfffffu) | L) != 0u) ? f_from(0x7fc00000u) : f_from(sign | 0x7f800000u);
     r.lo = 0.0f;
   }
+  return r;
+}
+// The same, with its range tests behind one that 2^-80 <= |x| < 2^128 pass: 20 instructions instead of 32
+GPSOC_DW DF dw_of(double x) {
+  const unsigned H = d_hi(x), L = d_lo(x);
+  const unsigned E = (H >> 20) & 0x7ffu;
+  if (E - 943u > 1149u - 943u) return dw_of_any(x);
+  const unsigned up = (L >> 28) & 1u;
+  DF r;
+  const unsigned s31 = H & 0x80000000u;   // E - 896, E - 919 and E - 942 are binary32 exponents
+  r.hi = f_from((s31 | ((E - 896u) << 23) | ((H & 0xfffffu) << 3) | (L >> 29)) + up);
+  const unsigned t1 = s31 | ((E - 919u) << 23), t2 = s31 | ((E - 942u) << 23);
+  const float a = rn_sub(f_from(t1 | ((L >> 6) & 0x7fffffu)), f_from(t1 + (up << 23)));
+  r.lo = rn_add(a, rn_sub(f_from(t2 | ((L & 0x3fu) << 17)), f_from(t2)));
   return r;
 }
 // binary64 -> binary32 by integer operations (the high word of dw_of: half-ulp ties up, values

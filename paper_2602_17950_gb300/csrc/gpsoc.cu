@@ -133,7 +133,8 @@ struct gpsoc_problem {
   double* d_part = nullptr;
   int pmax = 0;
   int nsm = 1;                  // SMs of the device (grid of the elementwise hybrid pass)
-  unsigned* d_cnt = nullptr;    // per-solve block arrival counters of the fused scalar steps
+  unsigned* d_cnt = nullptr;    // per-solve block arrival counters of the fused scalar steps, then of their groups
+  int gmax = 0;                 // group counters per solve
   double* d_scale = nullptr;    // per-solve scale factors
   double* d_tmp = nullptr;      // 3*batch doubles + model outputs
   size_t tmp_len = 0;
@@ -268,6 +269,8 @@ gpsoc_status chain_args(gpsoc_problem* p, int level, ChainArgs<T>& a) {
   a.gate = GATE_ACTIVE;
   a.scale = 1.0;
   a.cnt = p->d_cnt;
+  a.gcnt = p->d_cnt + p->batch;
+  a.gmax = p->gmax;
   if constexpr (sizeof(T) == 4) {
     for (int i = 0; i < p->dim; ++i) {
       gpsoc_status s = twiddles(p, a.g.n[i], &a.tw[i]);
@@ -569,6 +572,9 @@ HyArgs hy_args(gpsoc_problem* p, int level, const Geo& g, const ScalarCtx& sc, i
   h.p = p->b32.P[(parity & 1) ^ 1];   // direction of the previous iteration
   h.hlp = p->b32.HPhi;                // its H_lin P
   h.phi32 = p->b32.Phi;
+  h.philo = p->b32.D;                 // free in hybrid iterations
+  h.gcnt = p->d_cnt + p->batch;
+  h.gmax = p->gmax;
   h.hphi = p->b64.Z;                  // H(Phi): the FP64 Z buffer is free in hybrid iterations
   h.npts = g.npts;
   h.bps = hy_blocks_per_solve(g, p->batch, p->nsm);
@@ -692,7 +698,7 @@ gpsoc_status enqueue_iteration_hy(gpsoc_problem* p, int level, int parity, const
   ChainArgs<float> pi = a;
   pi.fuse = 1;
   pi.in0 = F.W; pi.in1 = F.G; pi.in2 = F.P[cur]; pi.in3 = F.Phi; pi.in4 = F.R[cur];
-  pi.phi64 = D.Phi; pi.out0 = F.HPhi; pi.out1 = nullptr;
+  pi.philo = F.D; pi.out0 = F.HPhi; pi.out1 = nullptr;
   RL<float>(p, ROW_INV_P_HY, pi);
   CK(cudaGetLastError());
   return GPSOC_OK;
@@ -1172,8 +1178,10 @@ gpsoc_status gpsoc_create(const gpsoc_grid* grid, const gpsoc_trap* trap, const 
   if (cudaMalloc(&p->d_part, sizeof(double) * (size_t)batch * NSLOT * p->pmax) != cudaSuccess)
     return bail(GPSOC_ENOMEM, "device allocation failed");
   if (cudaMalloc(&p->d_st, sizeof(SolveState) * batch) != cudaSuccess) return bail(GPSOC_ENOMEM, "device allocation failed");
-  if (cudaMalloc(&p->d_cnt, sizeof(unsigned) * batch) != cudaSuccess) return bail(GPSOC_ENOMEM, "device allocation failed");
-  if (cudaMemset(p->d_cnt, 0, sizeof(unsigned) * batch) != cudaSuccess) return bail(GPSOC_ECUDA, "memset failed");
+  p->gmax = (p->pmax + 63) / 64;   // groups of 64 blocks (group_sums)
+  const size_t cnt_bytes = sizeof(unsigned) * (size_t)batch * (1 + p->gmax);
+  if (cudaMalloc(&p->d_cnt, cnt_bytes) != cudaSuccess) return bail(GPSOC_ENOMEM, "device allocation failed");
+  if (cudaMemset(p->d_cnt, 0, cnt_bytes) != cudaSuccess) return bail(GPSOC_ECUDA, "memset failed");
   if (cudaMemset(p->d_st, 0, sizeof(SolveState) * batch) != cudaSuccess) return bail(GPSOC_ECUDA, "memset failed");
   if (cudaMallocHost(&p->h_st, sizeof(SolveState) * batch) != cudaSuccess) return bail(GPSOC_ENOMEM, "host allocation failed");
   if (cudaMalloc(&p->d_scale, sizeof(double) * batch) != cudaSuccess) return bail(GPSOC_ENOMEM, "device allocation failed");

@@ -187,9 +187,12 @@ struct ChainArgs {
   int given_r;        // ROW_FWD_PRE: in0 already holds r (mu taken as 0)
   int fuse;           // the last block of the pass runs the scalar step that consumes its sums
   unsigned* cnt;      // per-solve block arrival counters (fused scalar steps)
+  unsigned* gcnt;     // gmax group arrival counters per solve (group_sums)
+  int gmax;
   ScalarCtx sc;
   // GPSOC_HYBRID passes of an FP32 chain that also read the FP64 state
   const double2* phi64;   // Phi (FP64)
+  const C* philo;         // low words of Phi (the FP32 copy holds the high ones), for ROW_INV_P_HY
   const double2* hl64;    // H(Phi) (FP64), for ROW_FWD_PRE_HY
   // GPSOC_HYBRID, last column pass of the P chain: the spectrum of Phi (advanced by the
   // step applied this iteration when khat_upd is set) and of the previous P, both updated

@@ -73,15 +73,16 @@ __global__ void k_gather_obs(const SolveState* st, int batch, double* out) {
 // parameters (in the launch's own argument space: no copy from the host), cleared states and arrival counters.
 // With the observables taken in the last block of the last pass and small batches' states read whole, a
 // call is 4 launches and a copy instead of 6 launches and 4 copies: 73.4 -> 69.6 us for one 64^2 solve
-constexpr int kSetup = 64;
+constexpr int kSetup = 64;   // solves per launch
 struct SetupParams { PhysDev p[kSetup]; };
-__global__ void k_setup(SolveState* st, unsigned* cnt, PhysDev* phys, SetupParams q, int first, int count) {
+__global__ void k_setup(SolveState* st, unsigned* cnt, PhysDev* phys, SetupParams q, int first, int count,
+                        int counters) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= count) return;
   SolveState z{};
   z.active = 1;
   st[first + k] = z;
-  cnt[first + k] = 0u;
+  for (int i = 0; i < counters; ++i) cnt[(first + k) * counters + i] = 0u;
   phys[first + k] = q.p[k];
 }
 
@@ -132,6 +133,7 @@ extern "C" gpsoc_status gpsoc_apply_h_noalloc(const gpsoc_grid* grid, const gpso
   // 56 bytes a state and a table per axis are spare: part of the budget callers know
   const size_t o_st = off; off += align256((sizeof(SolveState) + 56) * batch);
   const size_t o_ph = off; off += align256(sizeof(PhysDev) * batch);
+  const size_t o_cnt = off;
   for (int i = 0; i < g.d; ++i) off += align256(sizeof(double2) * g.n[i]);
   const size_t o_obs = off; off += align256(sizeof(double) * 9 * batch);
   if (off > kNoAllocScratchBytes) {
@@ -149,9 +151,11 @@ extern "C" gpsoc_status gpsoc_apply_h_noalloc(const gpsoc_grid* grid, const gpso
   SolveState* sst = (SolveState*)(base + o_st);
   PhysDev* ph = (PhysDev*)(base + o_ph);
   double* dobs = (double*)(base + o_obs);
-  // set-up launches of kSetup solves; the arrival counters of the fused scalar step live where the gathered
-  // observables go afterwards
-  unsigned* cnt = (unsigned*)dobs;
+  // arrival counters of every solve's blocks and groups of 64 blocks: in the spare tables and, where many small
+  // solves need it, on into the place of the gathered observables, which are written after the last arrival
+  unsigned* cnt = (unsigned*)(base + o_cnt);
+  const int gmax = (pmax + 63) / 64;
+  if (sizeof(unsigned) * (size_t)batch * (1 + gmax) > off - o_cnt) return GPSOC_EBUDGET;   // 4 (1 + pmax / 64) of 72+ bytes
   for (int b0 = 0; b0 < batch; b0 += kSetup) {
     SetupParams q;
     const int nb = std::min(kSetup, batch - b0);
@@ -162,7 +166,7 @@ extern "C" gpsoc_status gpsoc_apply_h_noalloc(const gpsoc_grid* grid, const gpso
       }
       q.p[k] = make_phys(r.Omega, r.gamma, r.beta0, r.beta1);
     }
-    k_setup<<<1, kSetup, 0, st>>>(sst, cnt, ph, q, b0, nb);
+    k_setup<<<1, kSetup, 0, st>>>(sst, cnt, ph, q, b0, nb, 1 + gmax);
   }
   ChainArgs<double> a{};
   a.g = g;
@@ -177,6 +181,9 @@ extern "C" gpsoc_status gpsoc_apply_h_noalloc(const gpsoc_grid* grid, const gpso
   a.gate = GATE_ALL;
   a.nsolve = batch;
   a.scale = 1.0;
+  a.cnt = cnt;
+  a.gcnt = cnt + batch;
+  a.gmax = gmax;
   // the Hamiltonian chain of gpsoc_apply_h, on the caller's buffers and the scratch
   const double2* src = (const double2*)d_psi;
   a.in0 = src; a.out0 = A;
@@ -195,7 +202,6 @@ extern "C" gpsoc_status gpsoc_apply_h_noalloc(const gpsoc_grid* grid, const gpso
   // the last pass also takes E, mu, alpha and the masses from its sums
   a.in0 = W; a.in1 = G; a.in2 = src; a.out0 = (double2*)d_hpsi; a.out1 = nullptr;
   a.fuse = 1;
-  a.cnt = cnt;
   a.sc.st = sst; a.sc.phys = ph; a.sc.part = part; a.sc.pmax = pmax;
   a.sc.nb_row = nb_row;
   a.sc.nb_col = col_blocks_per_solve<double>(g, g.d - 1, batch);

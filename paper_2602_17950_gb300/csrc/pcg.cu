@@ -43,7 +43,7 @@ __global__ void k_scalar(ScalarArgs A) {
       return;
     case PH_NORM: {
       const int sl[1] = {SL_NORM};
-      slot_totals<double, 1, 1>(X, s, sl, A.nb_row, 0, -1, scratch);
+      slot_totals<double, 1, 1, true>(X, s, sl, A.nb_row, 0, -1, scratch);
       const double v = scratch[0];
       if (threadIdx.x == 0) A.norm_scale[s] = (v > 0.0 && isfinite(v)) ? 1.0 / sqrt(v * A.dV) : 0.0;
       return;
@@ -234,6 +234,7 @@ __global__ void __launch_bounds__(kHyThreads, kHyBlocksPerSM) k_hy_upd(HyArgs A)
       dwa_mul(acc[0], fy[c], hy[c]);
       dwa_add(acc[3 + c], m[c].hi, m[c].lo);
       A.phi32[at + c * npts] = make_float2(fx[c].hi, fy[c].hi);
+      A.philo[at + c * npts] = make_float2(fx[c].lo, fy[c].lo);
       mf[c] = fx[c].hi * fx[c].hi + fy[c].hi * fy[c].hi;   // the alpha pieces (FP32)
     }
     DF rho = m[0];
@@ -291,7 +292,12 @@ __global__ void __launch_bounds__(kHyThreads, kHyBlocksPerSM) k_hy_upd(HyArgs A)
     const double v = block_max((double)dmax, scratch);
     if (threadIdx.x == 0) put_partial(P + (long long)SL_DPHIINF * A.pmax, v, true, true);
   }
-  if (!red) return;
+  double* sums = A.part + (long long)s * NSLOT * A.pmax;
+  unsigned* gcnt = A.gcnt + (long long)s * A.gmax;
+  if (!red) {
+    if (dphi) group_max<DF>(sums, A.pmax, SL_DPHIINF, rb, bps, gcnt, scratch);
+    return;
+  }
   DF all[12];
 #pragma unroll
   for (int k = 0; k < 6; ++k) { all[k] = dwa_value(acc[k]); all[6 + k] = DF{acc32[k], 0.0f}; }
@@ -300,6 +306,7 @@ __global__ void __launch_bounds__(kHyThreads, kHyBlocksPerSM) k_hy_upd(HyArgs A)
   const int slots[12] = {SL_Q, SL_RHO2, SL_F2, SL_M0, SL_M1, SL_M2, SL_V0, SL_V1, SL_V2, SL_C0, SL_C1, SL_C2};
   const bool mx[12] = {};
   put_partials<12>(A.part, (long long)s * NSLOT, A.pmax, rb, slots, v, mx, true);
+  group_sums<DF, 12>(sums, A.pmax, slots, rb, bps, gcnt, scratch, dphi ? (int)SL_DPHIINF : -1);
 }
 
 // zero-pad the full spectrum of level N (in) into level 2N (out, zeroed first)

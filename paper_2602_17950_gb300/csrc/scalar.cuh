@@ -56,24 +56,36 @@ template <> struct TotOps<DF> {
   }
   static __device__ __forceinline__ double value(DF a) { return (double)a.hi + (double)a.lo; }
 };
+// A pass of more than kGroupFrom blocks per solve leaves one partial per group of kGroup blocks, at the
+// place of the group's first (group_sums): the scalar step of a 128^3 pass would otherwise read thousands,
+// 20 round trips to memory on one SM while the others wait (65 us of a 176 us row_inv_p_hy).
+constexpr int kGroup = 64, kGroupFrom = 1024;
+__host__ __device__ __forceinline__ int part_groups(int nb) { return (nb + kGroup - 1) / kGroup; }
+__device__ __forceinline__ int part_stride(int nb) { return nb > kGroupFrom ? kGroup : 1; }
+__device__ __forceinline__ int part_entries(int nb) { return nb > kGroupFrom ? part_groups(nb) : nb; }
+
+// sums of one warp's share: n0 entries (slots k < K0) or n1 from `base` on, st0 or st1 apart, dealt to the
+// threads tid < nt; the warp's sums go to scratch[warp * 32 + k]
 template <class V, int K, int K0>
-__device__ __forceinline__ void totals_of(const ScalarCtx& X, int s, const int (&slots)[K], int nb0, int nb1,
-                                          double* scratch) {
+__device__ __forceinline__ void totals_of(const double* base, int pmax, const int (&slots)[K], int n0, int st0, int n1,
+                                          int st1, int nt, double* scratch) {
   using O = TotOps<V>;
   constexpr int KP = (K <= 4) ? 4 : (K <= 8) ? 8 : (K <= 16) ? 16 : 32;
   constexpr int LB = (KP == 4) ? 2 : (KP == 8) ? 3 : (KP == 16) ? 4 : 5;
-  const double* base = X.part + (long long)s * NSLOT * X.pmax;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   V x[KP];
+  const double* p0 = base + (int)threadIdx.x * st0;
+  const double* p1 = base + (int)threadIdx.x * st1;
 #pragma unroll
   for (int k = 0; k < KP; ++k)
-    x[k] = (k < K && (int)threadIdx.x < (k < K0 ? nb0 : nb1))
-               ? O::load(base + (long long)slots[k < K ? k : 0] * X.pmax + threadIdx.x) : O::zero();
-  for (int b = threadIdx.x + blockDim.x; b < max(nb0, nb1); b += blockDim.x) {
+    x[k] = (k < K && (int)threadIdx.x < (k < K0 ? n0 : n1))
+               ? O::load((k < K0 ? p0 : p1) + (long long)slots[k < K ? k : 0] * pmax) : O::zero();
+  for (int b = threadIdx.x + nt; b < max(n0, n1); b += nt) {
     V t[K];
+    p0 += nt * st0;
+    p1 += nt * st1;
 #pragma unroll
-    for (int k = 0; k < K; ++k)
-      t[k] = b < (k < K0 ? nb0 : nb1) ? O::load(base + (long long)slots[k] * X.pmax + b) : O::zero();
+    for (int k = 0; k < K; ++k) t[k] = b < (k < K0 ? n0 : n1) ? O::load((k < K0 ? p0 : p1) + (long long)slots[k] * pmax) : O::zero();
 #pragma unroll
     for (int k = 0; k < K; ++k) x[k] = O::add(x[k], t[k]);
   }
@@ -95,17 +107,20 @@ __device__ __forceinline__ void totals_of(const ScalarCtx& X, int s, const int (
   for (int b = 0; b < LB; ++b) slot |= ((lane >> b) & 1) << (LB - 1 - b);
   if (lane < KP) scratch[warp * 32 + slot] = O::pack(x[0]);
 }
-template <class V, int K, int K0>
+// PLAIN: partials of an elementwise pass, which are not grouped
+template <class V, int K, int K0, bool PLAIN = false>
 __device__ __forceinline__ void slot_totals(const ScalarCtx& X, int s, const int (&slots)[K], int nb0, int nb1,
                                             int max_slot, double* scratch) {
   __shared__ unsigned long long s_max[32];
   const int nw = (blockDim.x + 31) >> 5;
-  totals_of<V, K, K0>(X, s, slots, nb0, nb1, scratch);
+  const double* base = X.part + (long long)s * NSLOT * X.pmax;
+  const int n0 = PLAIN ? nb0 : part_entries(nb0), st0 = PLAIN ? 1 : part_stride(nb0);
+  totals_of<V, K, K0>(base, X.pmax, slots, n0, st0, part_entries(nb1), part_stride(nb1), blockDim.x, scratch);
   if (max_slot >= 0) {
     unsigned long long m = 0;   // values that are not negative (or NaN) are ordered as their bits
-    const double* p = X.part + ((long long)s * NSLOT + max_slot) * X.pmax;
-    for (int b = threadIdx.x; b < nb0; b += blockDim.x) {
-      const unsigned long long v = (unsigned long long)__double_as_longlong(__ldcg(p + b));
+    const double* p = base + (long long)max_slot * X.pmax;
+    for (int b = threadIdx.x; b < n0; b += blockDim.x) {
+      const unsigned long long v = (unsigned long long)__double_as_longlong(__ldcg(p + (long long)b * st0));
       m = v > m ? v : m;
     }
     m = warp_max(m);
@@ -124,6 +139,50 @@ __device__ __forceinline__ void slot_totals(const ScalarCtx& X, int s, const int
     }
     __syncwarp();
   }
+}
+
+// The partials of block blk's group into one, by the last of its blocks to arrive: K sums (slots) and, if
+// max_slot >= 0, a maximum.  Every thread of every block calls it, once in a kernel (the counters know one
+// arrival per block), when the block's own partials are written; gcnt: the solve's group counters (zero;
+// they are left zero); scratch: 66 doubles.  Out of line: inlined it cost the passes that have no groups 2-3%.
+template <class V, int K>
+__device__ __noinline__ void group_sums_of(double* base, int pmax, const int* slots, int max_slot, int blk, int nb,
+                                           unsigned* gcnt, double* scratch) {
+  __shared__ int s_last;
+  const int g = blk / kGroup, n = min(kGroup, nb - g * kGroup);
+  if (!last_block(gcnt, g, n, &s_last)) return;
+  double* p = base + g * kGroup;
+  const int t = threadIdx.x;
+  if (max_slot >= 0 && t < kGroup) {
+    const unsigned long long m =
+        warp_max(t < n ? (unsigned long long)__double_as_longlong(__ldcg(p + (long long)max_slot * pmax + t)) : 0ull);
+    if ((t & 31) == 0) scratch[64 + (t >> 5)] = __longlong_as_double((long long)m);
+  }
+  // slot after slot (few registers): a warp adds 32 partials of a slot at a time
+  using O = TotOps<V>;
+  for (int k = t >> 5; k < 2 * K; k += blockDim.x >> 5) {
+    const int b = (k & 1) * 32 + (t & 31);
+    V x = b < n ? O::load(p + (long long)slots[k >> 1] * pmax + b) : O::zero();
+    for (int ofs = 16; ofs > 0; ofs >>= 1) x = O::add(x, O::shfl(x, ofs));
+    if ((t & 31) == 0) scratch[k] = O::pack(x);
+  }
+  __syncthreads();
+  if (t < K) p[(long long)slots[t] * pmax] = O::pack(O::add(O::from(scratch[2 * t]), O::from(scratch[2 * t + 1])));
+  if (max_slot >= 0 && t == 0) {
+    // as bits: a NaN stays the maximum
+    const long long m0 = __double_as_longlong(scratch[64]), m1 = __double_as_longlong(scratch[65]);
+    p[(long long)max_slot * pmax] = __longlong_as_double(m0 > m1 ? m0 : m1);
+  }
+}
+template <class V, int K>
+__device__ __forceinline__ void group_sums(double* base, int pmax, const int (&slots)[K], int blk, int nb, unsigned* gcnt,
+                                           double* scratch, int max_slot = -1) {
+  if (nb > kGroupFrom) group_sums_of<V, K>(base, pmax, slots, max_slot, blk, nb, gcnt, scratch);
+}
+template <class V>
+__device__ __forceinline__ void group_max(double* base, int pmax, int max_slot, int blk, int nb, unsigned* gcnt,
+                                          double* scratch) {
+  if (nb > kGroupFrom) group_sums_of<V, 0>(base, pmax, nullptr, max_slot, blk, nb, gcnt, scratch);
 }
 
 __device__ __forceinline__ void deactivate(SolveState& S, int status) {
@@ -216,8 +275,9 @@ __device__ __forceinline__ void sc_res(const ScalarCtx& X, int s, double* scratc
   SolveState& S = X.st[s];
   unsigned long long m = 0;
   const double* p = X.part + ((long long)s * NSLOT + SL_RINF) * X.pmax;
-  for (int b = threadIdx.x; b < X.nb_row; b += blockDim.x) {
-    const unsigned long long v = (unsigned long long)__double_as_longlong(__ldcg(p + b));
+  const int n = part_entries(X.nb_row), st = part_stride(X.nb_row);
+  for (int b = threadIdx.x; b < n; b += blockDim.x) {
+    const unsigned long long v = (unsigned long long)__double_as_longlong(__ldcg(p + (long long)b * st));
     m = v > m ? v : m;
   }
   m = warp_max(m);
