@@ -30,6 +30,9 @@ static constexpr int kThreads = 384;
 // reduction scratch (doubles) behind the tiles: block_reduce needs 16 per warp + 16
 static constexpr int kRedDoubles = 16 * (kThreads / 32) + 16;
 
+// elements per thread of the FP64 transforms of a tile of ept (see fft_lines)
+__device__ __forceinline__ int fx_ept(int ept, int n) { return (ept == 2 && n > 64) ? 4 : ept; }
+
 // Twiddle table in shared memory for transforms with E elements per thread:
 // entry (r, j) = W_n^(r j), r < E, j < n/E, at the padded index fft_pad(r n/E + j).
 // The last pass (radix E, Ns = n/E) reads j = k for consecutive groups k:
@@ -38,7 +41,7 @@ static constexpr int kRedDoubles = 16 * (kThreads / 32) + 16;
 template <class T>
 __device__ __forceinline__ void load_tw(cx_t<T>* s_tw, const cx_t<T>* tw, int n, int ept) {
   if constexpr (sizeof(T) == 8) {
-    fx_load_tw(reinterpret_cast<FxW*>(s_tw), n, ept == 8 ? 8 : 4, FftPad16{});
+    fx_load_tw(reinterpret_cast<FxW*>(s_tw), n, fx_ept(ept, n), FftPad16{});
   } else {
     const int lc = __ffs(n / ept) - 1;   // log2(n / E): n and E are powers of two
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -50,15 +53,17 @@ __device__ __forceinline__ void load_tw(cx_t<T>* s_tw, const cx_t<T>* tw, int n,
 
 // transforms of nlines lines at offset off (see fft_lines_e).  R16: the kernel may run radix-16 passes
 // (FP32 column passes only: the code path sets the register allocation of the whole kernel).
-// FP64 tiles of 2 elements per thread transform with half their threads.
+// FP64 tiles of 2 elements per thread transform lines of more than 64 points with half their threads, 4
+// elements each: radix-2 passes are twice as many and pay only where a solve is bound by the latency of
+// one warp per line (one 64^2 solve, 31 iterations: 3345 us with 4 elements, 3132 with 2).
 template <class C, bool R16 = false>
 __device__ __forceinline__ void fft_lines(int off, int nlines, int NP, int L, int ept, int down = 0) {
   if constexpr (R16 && sizeof(C) == 8) {
     if (ept == 16) { fft_lines_e<C, 16>(off, nlines, NP, L, down); return; }
   }
   if (ept == 8) fft_lines_e<C, 8>(off, nlines, NP, L, down);
-  else if (ept == 4 || sizeof(C) == 16) fft_lines_e<C, 4>(off, nlines, NP, L, down);
-  else if constexpr (sizeof(C) == 8) fft_lines_e<C, 2>(off, nlines, NP, L, down);
+  else if (ept == 4 || (sizeof(C) == 16 && L > 6)) fft_lines_e<C, 4>(off, nlines, NP, L, down);
+  else fft_lines_e<C, 2>(off, nlines, NP, L, down);
 }
 
 // padded length of a column line in shared memory

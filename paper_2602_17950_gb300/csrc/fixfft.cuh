@@ -75,13 +75,14 @@ constexpr FxTable fx_make_table() {
   return t;
 }
 
-// bits dropped by the twiddle product of a pass of E = 4 or 8 elements per thread, and bits F of a
+// bits dropped by the twiddle product of a pass of E = 2, 4 or 8 elements per thread, and bits F of a
 // line's values before a first pass of radix R
-template <int E> constexpr int kFxShift = (E == 8) ? 3 : 2;
+template <int E> constexpr int kFxShift = (E == 8) ? 3 : (E == 4) ? 2 : 1;
 template <int R> constexpr int kFxBits = 62 - ((R == 8) ? 3 : (R == 4) ? 2 : 1);
 
-// table entry (units of 2^-62) as the split twiddle in units of 2^-(64 - shift); the low half
-// stays above -2^31, so that its negative is an int too
+// table entry (units of 2^-62) as the split twiddle in units of 2^-(64 - shift), shift 2 or 3 (E = 2: 2, as
+// units of 2^-63 would not hold w = 1, and fx_cmul doubles its product); the low half stays above -2^31, so
+// that its negative is an int too
 GPSOC_FX void fx_split(long long w, int shift, int& hi, int& lo) {
   long long v = (w + ((1LL << (shift - 2)) >> 1)) >> (shift - 2);
   lo = (int)(unsigned)v;
@@ -183,18 +184,23 @@ GPSOC_FX void fx_halves(long long a, int& h, int& l) {
   h = (int)(a >> 32) + (int)((unsigned)a >> 31);
 }
 // a w 2^-shift for a complex value below 2^62.5 and a split twiddle (conj: its conjugate).  The
-// product of the low halves is left out (below one unit), the middle ones are rounded.
-template <bool CONJ>
+// product of the low halves is left out (below one unit), the middle ones are rounded.  TWICE: 2 a w 2^-shift.
+template <bool CONJ, bool TWICE = false>
 GPSOC_FX FxC fx_cmul(FxC a, FxW w) {
   int xh, xl, yh, yl;
   fx_halves(a.x, xh, xl);
   fx_halves(a.y, yh, yl);
   const int ph = CONJ ? w.yh : -w.yh, pl = CONJ ? w.yl : -w.yl;   // of a.y in the real part
   const int qh = -ph, ql = -pl;                                     // of a.x in the imaginary part
-  const long long half = 1LL << 31;
+  const long long half = TWICE ? 1LL << 30 : 1LL << 31;
   const long long mr = half + (long long)xh * w.xl + (long long)xl * w.xh + (long long)yh * pl + (long long)yl * ph;
   const long long mi = half + (long long)yh * w.xl + (long long)yl * w.xh + (long long)xh * ql + (long long)xl * qh;
   FxC r;
+  if (TWICE) {
+    r.x = (mr >> 31) + 2 * ((long long)xh * w.xh + (long long)yh * ph);
+    r.y = (mi >> 31) + 2 * ((long long)yh * w.xh + (long long)xh * qh);
+    return r;
+  }
   r.x = (mr >> 32) + (long long)xh * w.xh + (long long)yh * ph;
   r.y = (mi >> 32) + (long long)yh * w.xh + (long long)xh * qh;
   return r;
@@ -265,7 +271,7 @@ template <bool INV, int R> GPSOC_FX void fx_dft(FxC* v) {
 __device__ const FxTable g_fx_table = fx_make_table();
 
 // Twiddles for transforms of length n with E elements per thread: entry (r, j) = W_n^(r j) 2^-shift,
-// r < E, j < n/E, at the padded index pad(r n/E + j).  E = 4 or 8.
+// r < E, j < n/E, at the padded index pad(r n/E + j).
 template <class Pad>
 __device__ __forceinline__ void fx_load_tw(FxW* s_tw, int n, int ept, Pad pad) {
   const int lc = __ffs(n / ept) - 1, step = kFxTable / n, shift = (ept == 8) ? 3 : 2;
@@ -351,7 +357,7 @@ __device__ __forceinline__ void fx_pass(FxC* p, bool act, int g0, int N, int Ns,
         const int j = k * (N / (Ns * R));
         v[u * R] = fx_shift(v[u * R], kFxShift<E>);
 #pragma unroll
-        for (int r = 1; r < R; ++r) v[u * R + r] = fx_cmul<false>(v[u * R + r], tw[pad(r * G + j)]);
+        for (int r = 1; r < R; ++r) v[u * R + r] = fx_cmul<false, E == 2>(v[u * R + r], tw[pad(r * G + j)]);
       }
       fx_dft<false, R>(&v[u * R]);
       const int ob = (g - k) * R + k;
@@ -386,7 +392,7 @@ template <int E, class Pad>
 __device__ __forceinline__ void fx_fft(FxC* p, bool act, int g0, int L, int down, const FxW* tw, int* s_key, bool warp,
                                        Pad pad) {
   const int N = 1 << L;
-  constexpr int LE = (E == 8) ? 3 : 2;
+  constexpr int LE = (E == 8) ? 3 : (E == 4) ? 2 : 1;
   const int rem = L % LE, full = L / LE;
   int Ns = E, n = 1, sc = 0;
   if (rem == 1) { fx_pass<2, E, true>(p, act, g0, N, 1, tw, full == 0, sc, down, s_key, warp, pad); Ns = 2; n = 0; }

@@ -29,9 +29,9 @@ static void pass(const FxC* in, FxC* out, int n, int Ns, bool first) {
       }
       const int at = r * k * (n / (Ns * R)) * (kFxTable / n);
       FxW w;
-      fx_split(g_table.c[2 * at], shift, w.xh, w.xl);
-      fx_split(g_table.c[2 * at + 1], shift, w.yh, w.yl);
-      v[r] = fx_cmul<INV>(v[r], w);
+      fx_split(g_table.c[2 * at], E == 8 ? 3 : 2, w.xh, w.xl);
+      fx_split(g_table.c[2 * at + 1], E == 8 ? 3 : 2, w.yh, w.yl);
+      v[r] = fx_cmul<INV, E == 2>(v[r], w);
     }
     fx_dft<INV, R>(v);
     for (int q = 0; q < R; ++q) out[(g - k) * R + k + q * Ns] = v[q];
@@ -43,7 +43,7 @@ static void line(double* d, int n) {
   int key = 0;
   for (int i = 0; i < 2 * n; ++i) key = fx_key(d[i]) > key ? fx_key(d[i]) : key;
   const int em = (key >> 20) > 1 ? key >> 20 : 1;
-  constexpr int LE = (E == 8) ? 3 : 2;
+  constexpr int LE = (E == 8) ? 3 : (E == 4) ? 2 : 1;
   int L = 0;
   while ((1 << L) < n) ++L;
   const int rem = L % LE, lr = rem ? rem : LE;
@@ -53,7 +53,7 @@ static void line(double* d, int n) {
   for (int i = 0; i < n; ++i) { a[i].x = fx_of(d[2 * i], em, F); a[i].y = fx_of(d[2 * i + 1], em, F); }
   int sc = em - 1022 - F, Ns = 1 << lr;
   if (lr == 1) pass<INV, 2, E>(a, b, n, 1, true);
-  else if (lr == 2) pass<INV, 4, E>(a, b, n, 1, true);
+  else if (lr == 2) pass<INV, (E >= 4 ? 4 : 2), E>(a, b, n, 1, true);
   else pass<INV, E, E>(a, b, n, 1, true);
   for (; Ns < n; Ns *= E) {
     FxC* t = a; a = b; b = t;
@@ -69,10 +69,11 @@ static void line(double* d, int n) {
 }
 
 extern "C" {
-// in place, unnormalised, n a power of two in [8, 1024], E = 4 or 8
+// in place, unnormalised, n a power of two in [8, 1024], E = 2, 4 or 8
 void fx_line(double* d, int n, int e, int inverse) {
   if (e == 8) inverse ? line<true, 8>(d, n) : line<false, 8>(d, n);
-  else inverse ? line<true, 4>(d, n) : line<false, 4>(d, n);
+  else if (e == 4) inverse ? line<true, 4>(d, n) : line<false, 4>(d, n);
+  else inverse ? line<true, 2>(d, n) : line<false, 2>(d, n);
 }
 // table entry k as (re, im) in units of 2^-62
 void fx_table(int k, long long* out) { out[0] = g_table.c[2 * k]; out[1] = g_table.c[2 * k + 1]; }

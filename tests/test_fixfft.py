@@ -47,7 +47,7 @@ def _exact(x, inverse=False):
 
 def _fp64(x, e, inverse=False):
     """FP64 Stockham passes in the order of the transforms tested."""
-    n, L, le = len(x), int(np.log2(len(x))), {4: 2, 8: 3}[e]
+    n, L, le = len(x), int(np.log2(len(x))), {2: 1, 4: 2, 8: 3}[e]
     rem, y, ns = L % le, x.astype(np.complex128), 1
     sgn = 1 if inverse else -1
     radices = ([2 ** rem] if rem else []) + [e] * (L // le)
@@ -119,8 +119,9 @@ def test_conversions(lib):
     assert lib.fx_widen(1 << 40, 1000) == np.inf and lib.fx_widen(-(1 << 40), -1200) == 0.0
 
 
-@pytest.mark.parametrize("n", [8, 16, 32, 64, 128, 256, 512, 1024])
-@pytest.mark.parametrize("e", [4, 8])
+# 2 elements per thread: lines of up to 64 points only
+@pytest.mark.parametrize("n,e", [(n, e) for e in (4, 8) for n in (8, 16, 32, 64, 128, 256, 512, 1024)]
+                         + [(n, 2) for n in (8, 16, 32, 64)])
 def test_lines_no_less_exact_than_fp64(lib, n, e):
     for inverse in (False, True):
         for name, x in _inputs(n, n + e).items():
