@@ -538,7 +538,7 @@ enum RowMode {
   ROW_FWD_PRE_HY,      // FP32 pass of GPSOC_HYBRID: r = H Phi - mu Phi in FP64 from phi64 and H(Phi)
                        // (hl64) -> out1 (FP32); out0 = F_x(P_V^{1/2} r); reduce max|r|
   ROW_INV_P_HY         // FP32 pass of GPSOC_HYBRID: as ROW_INV_P with in4 = r (slot HPHIP = Re<r, P>),
-                       // out0 = H_lin P, and Re<P, Phi> summed in FP64 against phi64
+                       // out0 = H_lin P, and the step integrals with Phi = FP32 copy + low words
 };
 enum ColMode {
   COL_FWD = 0,         // out0 = F_axis(in0)
