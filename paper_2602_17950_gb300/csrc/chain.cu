@@ -791,6 +791,23 @@ template <class T> void tuned(const Geo& g, int axis, int nsolve, int& lines, in
 }
 }  // namespace
 
+template <class T> bool tile_valid(const Geo& g, int axis, int lines, int ept);
+
+// elements per thread of the FFT passes: 16 (radix-16 passes, FP32 column passes) or 8,
+// unless the tile would then have fewer than 128 threads or a line is shorter,
+// in which case fewer (more threads, more passes); and the matching thread
+// count (multiple of 32, >= 64).  Rows: where the blocks fill the SMs, 8 (FP32: 16 x 64^2 hybrid
+// 1493 us with 2, 1386 with 8) or at least 4 (FP64: 16 x 64^2 3118 us with 2, 3013 with 4) whatever the threads.
+template <class T>
+static int pick_ept(int work /* complex elements of the three components */, int n /* line length */, bool column,
+                    long long blocks) {
+  int e = (sizeof(T) == 4 && column) ? 16 : 8;
+  const bool full = !column && blocks >= kTargetBlocks;
+  const int least = full ? (sizeof(T) == 4 ? 8 : 4) : 2;
+  while (e > 2 && ((work / e < 128 && e > least) || e > n)) e >>= 1;
+  return e;
+}
+
 template <class T>
 int row_rows_per_block(const Geo& g, int nsolve) {
   int tl, te;
@@ -823,23 +840,12 @@ int col_tc(const Geo& g, int axis, int nsolve) {
     if (tc < 4) tc = ni < 4 ? ni : 4;
     else if (2 * tc <= ni && 2 * tc * na <= 2048 && columns / (2 * tc) >= 4 * kTargetBlocks) tc *= 2;
   }
+  // no more than the kernels run: 4 columns of 1024 points are 768 threads, as are 256 of 8 points (one 1024^2
+  // hybrid iteration: 617 us with the 2 columns this leaves, 738 with 1)
+  while (tc > 1 && !tile_valid<T>(g, axis, tc, pick_ept<T>(3 * tc * na, na, true, 0))) tc >>= 1;
   return tc;
 }
 
-// elements per thread of the FFT passes: 16 (radix-16 passes, FP32 column passes) or 8,
-// unless the tile would then have fewer than 128 threads or a line is shorter,
-// in which case fewer (more threads, more passes); and the matching thread
-// count (multiple of 32, >= 64).  Rows: where the blocks fill the SMs, 8 (FP32: 16 x 64^2 hybrid
-// 1493 us with 2, 1386 with 8) or at least 4 (FP64: 16 x 64^2 3118 us with 2, 3013 with 4) whatever the threads.
-template <class T>
-static int pick_ept(int work /* complex elements of the three components */, int n /* line length */, bool column,
-                    long long blocks) {
-  int e = (sizeof(T) == 4 && column) ? 16 : 8;
-  const bool full = !column && blocks >= kTargetBlocks;
-  const int least = full ? (sizeof(T) == 4 ? 8 : 4) : 2;
-  while (e > 2 && ((work / e < 128 && e > least) || e > n)) e >>= 1;
-  return e;
-}
 static int round_threads(int t) {
   if (t < 64) t = 64;
   return (t + 31) & ~31;
