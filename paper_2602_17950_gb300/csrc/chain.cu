@@ -211,7 +211,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           f[c] = A.in0[at + c * npts];
-          if (upd) p[c] = __ldg(A.in2 + at + c * npts);
+          if (upd) p[c] = A.in2[at + c * npts];
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -231,9 +231,9 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
         C z[3], f[3], q[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          z[c] = __ldg(A.in0 + at + c * npts);
-          f[c] = __ldg(A.in1 + at + c * npts);
-          q[c] = use_prev ? __ldg(A.in2 + at + c * npts) : mk<C>((W)0, (W)0);
+          z[c] = A.in0[at + c * npts];
+          f[c] = A.in1[at + c * npts];
+          q[c] = use_prev ? A.in2[at + c * npts] : mk<C>((W)0, (W)0);
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -255,8 +255,8 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
         double2 f[3], h[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          f[c] = __ldg(A.phi64 + at + c * npts);
-          h[c] = __ldg(A.hl64 + at + c * npts);
+          f[c] = A.phi64[at + c * npts];
+          h[c] = A.hl64[at + c * npts];
         }
         W rho = (W)0;
 #pragma unroll
@@ -279,8 +279,8 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
         C f[3], h[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          f[c] = __ldg(A.in1 + at + c * npts);
-          h[c] = __ldg(A.in0 + at + c * npts);
+          f[c] = A.in1[at + c * npts];
+          h[c] = A.in0[at + c * npts];
         }
         W rho = (W)0;
 #pragma unroll
@@ -354,11 +354,11 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
       C f[3], rr[3], rp[3], pp[3];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        f[c] = __ldg(A.in1 + at + c * npts);
-        rr[c] = __ldg(A.in2 + at + c * npts);
+        f[c] = A.in1[at + c * npts];
+        rr[c] = A.in2[at + c * npts];
         if (use_prev) {
-          rp[c] = __ldg(A.in3 + at + c * npts);
-          pp[c] = __ldg(A.in4 + at + c * npts);
+          rp[c] = A.in3[at + c * npts];
+          pp[c] = A.in4[at + c * npts];
         }
       }
 #pragma unroll
@@ -405,12 +405,12 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
     C fl[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      u[c] = __ldg(A.in2 + at + c * npts);
+      u[c] = A.in2[at + c * npts];
       if (MODE == ROW_INV_P || MODE == ROW_INV_P_HY) {
-        f[c] = __ldg(A.in3 + at + c * npts);
-        h[c] = __ldg(A.in4 + at + c * npts);
+        f[c] = A.in3[at + c * npts];
+        h[c] = A.in4[at + c * npts];
       }
-      if (MODE == ROW_INV_P_HY) fl[c] = __ldg(A.philo + at + c * npts);
+      if (MODE == ROW_INV_P_HY) fl[c] = A.philo[at + c * npts];
     }
     const W ox = Omn * coord<W>(A.g, 0, j);
     const W V = trap_value<W>(A.trap, A.g, j, row & (ny - 1), row >> Ly, at - (long long)s * 3 * npts);
@@ -721,7 +721,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_col(ChainArgs<T> A, int axis, i
       const W rot = rx * coord<W>(A.g, 1, j);
       C a[3];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) a[c] = __ldg((MODE == COL_YINV_H ? A.in1 : A.in0) + at + c * npts);
+      for (int c = 0; c < 3; ++c) a[c] = (MODE == COL_YINV_H ? A.in1 : A.in0)[at + c * npts];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const C v = buf[sidx(c, jr)], gv = buf2[sidx(c, jr)];

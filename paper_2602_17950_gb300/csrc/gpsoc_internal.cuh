@@ -205,7 +205,8 @@ struct ChainArgs {
 // (launch_pdl): once every block of a kernel has exited, the blocks of the next one are placed before
 // the kernel counts as complete and its writes are visible.  They set up what no kernel writes
 // (twiddles) and stop at pdl_wait() (griddepcontrol.wait) until then; every read of data another
-// kernel writes comes after it.  12 us of the 83 us H(Phi) of 64^2, 5 us of the 75 us of a 128^2
+// kernel writes comes after it, as an ordinary load: __ldg is for data that is constant from a kernel's launch
+// on, and the compiler need not keep it behind the wait.  12 us of the 83 us H(Phi) of 64^2, 5 us of the 75 us of a 128^2
 // hybrid iteration.  Triggering the next kernel earlier (griddepcontrol.launch_dependents after a
 // block's own wait) placed its blocks around the running ones, on fewer SMs: 256^2 hybrid 1422 -> 1743 us.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

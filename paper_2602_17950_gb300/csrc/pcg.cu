@@ -183,8 +183,8 @@ __global__ void __launch_bounds__(kHyThreads, kHyBlocksPerSM) k_hy_upd(HyArgs A)
     for (int c = 0; c < 3; ++c) {
       f64[c] = A.phi[at + c * npts];
       if (red || rec) h64[c] = A.hl[at + c * npts];
-      if (upd) q[c] = __ldg(A.p + at + c * npts);
-      if (rec) hq[c] = __ldg(A.hlp + at + c * npts);
+      if (upd) q[c] = A.p[at + c * npts];
+      if (rec) hq[c] = A.hlp[at + c * npts];
     }
     DF fx[3], fy[3], hx[3], hy[3];
 #pragma unroll
