@@ -1804,7 +1804,7 @@ gpsoc_status load_slot(Bucket* b, int s, const ServerReq& r) {
 
 // The slots loaded since the last call: parameters, normalisation and PCG state (first = 1 restarts
 // beta), all of them in one set of launches (12 requests of 64^2, submission to last answer: 2210 us with a
-// set for each, 2139 with one).
+// set for each, 2139 with one).  The caller empties the list.
 gpsoc_status init_slots(Bucket* b) {
   gpsoc_problem* p = b->p;
   const Geo g = make_geo(p, 0);
@@ -1841,7 +1841,6 @@ gpsoc_status init_slots(Bucket* b) {
     }
   }
   CK(cudaGetLastError());
-  b->fresh.clear();
   return GPSOC_OK;
 }
 
@@ -2060,26 +2059,30 @@ gpsoc_status server_step_impl(gpsoc_server* s, int* busy, bool bounded, Clock::t
   }
   // 2. admission: fill free slots from the queue, in arrival order (a slot load is
   //    stream-ordered after any round still running in its bucket)
+  // an error ends admission: what it met stays queued with those behind it, what was admitted runs
   std::vector<uint64_t> waiting;
-  for (uint64_t t : s->queue) {
+  for (size_t i = 0; i < s->queue.size(); ++i) {
+    const uint64_t t = s->queue[i];
     ServerReq* r = s->reqs[t];
-    Bucket* b = find_or_make_bucket(s, *r, r->stage, &err);
-    if (err != GPSOC_OK) break;
+    Bucket* b = err == GPSOC_OK ? find_or_make_bucket(s, *r, r->stage, &err) : nullptr;
     if (!b) { waiting.push_back(t); continue; }
     int slot = -1;
     for (size_t k = 0; k < b->slot.size(); ++k)
       if (b->slot[k] < 0) { slot = (int)k; break; }
     err = load_slot(b, slot, *r);
-    if (err != GPSOC_OK) break;
+    if (err != GPSOC_OK) { waiting.push_back(t); continue; }
     b->slot[slot] = (int64_t)t;
   }
-  for (Bucket* b : s->buckets) {     // also those loaded before an error
+  for (Bucket* b : s->buckets) {
     if (b->fresh.empty()) continue;
     const gpsoc_status st = init_slots(b);
+    if (st != GPSOC_OK)                // their slots are given back
+      for (int k : b->fresh) { waiting.push_back((uint64_t)b->slot[k]); b->slot[k] = -1; }
+    b->fresh.clear();
     if (err == GPSOC_OK) err = st;
   }
-  if (err != GPSOC_OK) return err;
   s->queue.swap(waiting);
+  if (err != GPSOC_OK) return err;
   // 3. every idle bucket that holds work starts its next round on its own stream
   const int iters = s->opts.iters_per_step > 0 ? s->opts.iters_per_step : 32;
   const int pairs = (iters + 1) / 2;
