@@ -8,8 +8,8 @@
 // building blocks of double-word arithmetic" (ACM TOMS 2017): the accurate double-word sum
 // (TwoSum of the high and of the low parts, two FastTwoSum renormalisations; relative
 // error below 3u^2, u = 2^-24) and the FMA-based products, double word x double word
-// without the lo x lo term and double word x binary32, with relative errors of a few u^2
-// (the CPU checks bound them by 7u^2 and 4u^2).  Every step is an
+// without the lo x lo term (its cross products in one chain of FMAs) and double word x
+// binary32, with relative errors of a few u^2 (the CPU checks bound them by 7u^2 and 4u^2).  Every step is an
 // explicit round-to-nearest operation, so multiply-add contraction cannot break the
 // error-free transformations.  Conversions to and from binary64 move the fields of the
 // IEEE 754 encodings with integer operations (one FP64 add per value stored back).
@@ -140,8 +140,11 @@ GPSOC_DW DF dw_sub(DF a, DF b) { return dw_add(a, dw_neg(b)); }
 GPSOC_DW DF dw_mul(DF a, DF b) {
   const float ch = rn_mul(a.hi, b.hi);
   const float cl = rn_fma(a.hi, b.hi, -ch);                       // TwoProd: a.hi b.hi = ch + cl
-  const float t = rn_fma(a.lo, b.hi, rn_mul(a.hi, b.lo));
-  return dw_fast_two_sum(ch, rn_add(cl, t));
+  return dw_fast_two_sum(ch, rn_fma(a.lo, b.hi, rn_fma(a.hi, b.lo, cl)));
+}
+GPSOC_DW DF dw_sqr(DF a) {
+  const float ch = rn_mul(a.hi, a.hi);
+  return dw_fast_two_sum(ch, rn_fma(a.hi + a.hi, a.lo, rn_fma(a.hi, a.hi, -ch)));
 }
 GPSOC_DW DF dw_mulf(DF a, float b) {
   const float ch = rn_mul(a.hi, b);
@@ -215,48 +218,27 @@ GPSOC_DW float narrow_f(double x) {
   if (E > 1150) u = (E == 2047 && ((H & 0xfffffu) | L) != 0u) ? 0x7fc00000u : (sign | 0x7f800000u);
   return f_from(u);
 }
-// Running sums of products in a double word that is normalised once, at the end (dwa_value): the high
-// word takes each product's leading part exactly (TwoSum), the low word the parts it leaves and the
-// products' own error terms.  Relative to the sum of the terms' moduli the error is a few u^2 as with
-// dw_add and dw_mul for every term, at 9 to 12 instructions a term instead of 28.
+// Sums of products in a double word: each product is normalised, added with one TwoSum of the high words,
+// and the sum normalised again: 18 instructions a term against 28 with dw_add and the product it
+// takes.  Errors are relative to the terms' moduli (dw_add's to the sum, also where terms cancel), so these are
+// for two or three terms that are new; a state or a total takes them with dw_add (hypoint.cuh).  Normalising once,
+// at the end of a sum, is 11 instructions a term, but its error is up to 2.7 times as large.
 GPSOC_DW void dwa_add(DF& A, float p, float e) {
   const DF s = dw_two_sum(A.hi, p);
-  A.hi = s.hi;
-  A.lo = rn_add(A.lo, rn_add(s.lo, e));
+  A = dw_fast_two_sum(s.hi, rn_add(s.lo, rn_add(A.lo, e)));
 }
-GPSOC_DW void dwa_sq(DF& A, float a) {               // += a a
+GPSOC_DW void dwa_sum(DF& A, DF a) { dwa_add(A, a.hi, a.lo); }                       // += a
+GPSOC_DW void dwa_mul(DF& A, DF a, DF b) { dwa_sum(A, dw_mul(a, b)); }               // += a b
+GPSOC_DW void dwa_sub(DF& A, DF a, DF b) { dwa_sum(A, dw_mul(dw_neg(a), b)); }       // -= a b
+GPSOC_DW void dwa_mulf(DF& A, DF a, float b) { dwa_sum(A, dw_mulf(a, b)); }          // += a b
+GPSOC_DW void dwa_sqd(DF& A, DF a) { dwa_sum(A, dw_sqr(a)); }                        // += a a
+GPSOC_DW void dwa_sq(DF& A, float a) {                                               // += a a
   const float p = rn_mul(a, a);
   dwa_add(A, p, rn_fma(a, a, -p));
 }
-GPSOC_DW void dwa_mulf(DF& A, DF a, float b) {       // += a b
-  const float p = rn_mul(a.hi, b);
-  dwa_add(A, p, rn_fma(a.lo, b, rn_fma(a.hi, b, -p)));
-}
-GPSOC_DW void dwa_mul(DF& A, DF a, DF b) {           // += a b
-  const float p = rn_mul(a.hi, b.hi);
-  dwa_add(A, p, rn_fma(a.lo, b.hi, rn_fma(a.hi, b.lo, rn_fma(a.hi, b.hi, -p))));
-}
-GPSOC_DW void dwa_sub(DF& A, DF a, DF b) {           // -= a b
-  const float p = rn_mul(-a.hi, b.hi);
-  dwa_add(A, p, rn_fma(-a.lo, b.hi, rn_fma(-a.hi, b.lo, rn_fma(-a.hi, b.hi, -p))));
-}
-GPSOC_DW void dwa_sqd(DF& A, DF a) {                 // += a a
-  const float p = rn_mul(a.hi, a.hi);
-  dwa_add(A, p, rn_fma(a.hi + a.hi, a.lo, rn_fma(a.hi, a.hi, -p)));
-}
-GPSOC_DW DF dwa_of_mul(DF a, DF b) {                 // a sum that opens with a b
-  DF r;
-  r.hi = rn_mul(a.hi, b.hi);
-  r.lo = rn_fma(a.lo, b.hi, rn_fma(a.hi, b.lo, rn_fma(a.hi, b.hi, -r.hi)));
-  return r;
-}
-GPSOC_DW DF dwa_of_sqd(DF a) {
-  DF r;
-  r.hi = rn_mul(a.hi, a.hi);
-  r.lo = rn_fma(a.hi + a.hi, a.lo, rn_fma(a.hi, a.hi, -r.hi));
-  return r;
-}
-GPSOC_DW DF dwa_value(DF A) { return dw_fast_two_sum(A.hi, A.lo); }
+GPSOC_DW DF dwa_of_mul(DF a, DF b) { return dw_mul(a, b); }                          // a sum that opens with a b
+GPSOC_DW DF dwa_of_sqd(DF a) { return dw_sqr(a); }
+GPSOC_DW DF dwa_value(DF A) { return A; }
 
 // double word -> binary64, correctly rounded: one FP64 add of the two exact widenings
 GPSOC_DW double dw_to_double(DF a) { return widen_f(a.hi) + widen_f(a.lo); }

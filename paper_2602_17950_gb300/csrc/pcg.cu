@@ -12,6 +12,7 @@
 #include <algorithm>
 
 #include "gpsoc_internal.cuh"
+#include "hypoint.cuh"
 #include "kernels.cuh"
 #include "scalar.cuh"
 
@@ -197,87 +198,35 @@ __global__ void __launch_bounds__(kHyThreads, kHyBlocksPerSM) k_hy_upd(HyArgs A)
       }
       if (upd) {
         // the accepted step (Eqs. formula-pcg, update) with the exact tangent direction
-        if (dphi) {
-          const float dx = ucm1.hi * fx[c].hi + ut.hi * q[c].x, dy = ucm1.hi * fy[c].hi + ut.hi * q[c].y;
-          dmax = fmaxf(dmax, dx * dx + dy * dy);
-        }
-        DF nx_ = dwa_of_mul(ucm1, fx[c]), ny_ = dwa_of_mul(ucm1, fy[c]);
-        dwa_mulf(nx_, ut, q[c].x);
-        dwa_mulf(ny_, ut, q[c].y);
-        dwa_add(nx_, fx[c].hi, fx[c].lo);
-        dwa_add(ny_, fy[c].hi, fy[c].lo);
-        fx[c] = dwa_value(nx_);
-        fy[c] = dwa_value(ny_);
+        const DF dx = hy_change(ucm1, ut, fx[c], q[c].x), dy = hy_change(ucm1, ut, fy[c], q[c].y);
+        if (dphi) dmax = fmaxf(dmax, dx.hi * dx.hi + dy.hi * dy.hi);
+        fx[c] = dw_add(fx[c], dx);
+        fy[c] = dw_add(fy[c], dy);
         A.phi[at + c * npts] = make_double2(dw_to_double(fx[c]), dw_to_double(fy[c]));
         if (rec) {
           // H_lin is linear: H_lin Phi' = g (c H_lin Phi + t H_lin P)
-          DF gx = dwa_of_mul(uc, hx[c]), gy = dwa_of_mul(uc, hy[c]);
-          dwa_mulf(gx, ut, hq[c].x);
-          dwa_mulf(gy, ut, hq[c].y);
-          hx[c] = dwa_value(gx);
-          hy[c] = dwa_value(gy);
+          hx[c] = hy_linear(uc, ut, hx[c], hq[c].x);
+          hy[c] = hy_linear(uc, ut, hy[c], hq[c].y);
           A.hl[at + c * npts] = make_double2(dw_to_double(hx[c]), dw_to_double(hy[c]));
         }
       }
     }
     if (!red) continue;
-    // H(Phi) = H_lin Phi + c0 rho Phi + c1 (F.f) Phi (Eqs. eigen1-eigen3) and the sums of the
-    // energy (Eq. energy) and of alpha_l (Eq. PreCnstAlpha)
-    DF m[3];
+    // H(Phi) and the sums of the energy (Eq. energy) and of alpha_l (Eq. PreCnstAlpha)
+    const HyPoint pt = hy_point(fx, fy);
+    hy_sums(acc, pt, fx, fy, hx, hy);
     float mf[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      DF t = dwa_of_sqd(fx[c]);
-      dwa_sqd(t, fy[c]);
-      m[c] = dwa_value(t);
-      dwa_mul(acc[0], fx[c], hx[c]);
-      dwa_mul(acc[0], fy[c], hy[c]);
-      dwa_add(acc[3 + c], m[c].hi, m[c].lo);
       A.phi32[at + c * npts] = make_float2(fx[c].hi, fy[c].hi);
       A.philo[at + c * npts] = make_float2(fx[c].lo, fy[c].lo);
       mf[c] = fx[c].hi * fx[c].hi + fy[c].hi * fy[c].hi;   // the alpha pieces (FP32)
     }
-    DF rho = m[0];
-    dwa_add(rho, m[1].hi, m[1].lo);
-    dwa_add(rho, m[2].hi, m[2].lo);
-    rho = dwa_value(rho);
-    // a = phi_1 conj(phi_0) + phi_0 conj(phi_-1) (components ordered 1, 0, -1), Fz = |phi_1|^2 - |phi_-1|^2
-    DF ar = dwa_of_mul(fx[1], fx[0]), ai = dwa_of_mul(fx[1], fy[0]);
-    dwa_mul(ar, fy[1], fy[0]);
-    dwa_mul(ar, fx[2], fx[1]);
-    dwa_mul(ar, fy[2], fy[1]);
-    dwa_sub(ai, fy[1], fx[0]);
-    dwa_mul(ai, fx[2], fy[1]);
-    dwa_sub(ai, fy[2], fx[1]);
-    ar = dwa_value(ar);
-    ai = dwa_value(ai);
-    DF Fz = m[0];
-    dwa_add(Fz, -m[2].hi, -m[2].lo);
-    Fz = dwa_value(Fz);
-    const DF c0r = dw_mul(c0, rho), cz = dw_mul(c1, Fz), cr = dw_mul(c1, ar), ci = dw_mul(c1, ai);
-    // each component of H in one sum; rounded to FP64 from there
     DF h[6];
+    hy_hamiltonian(pt, c0, c1, fx, fy, hx, hy, h);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      h[2 * c] = dwa_of_mul(c0r, fx[c]);
-      h[2 * c + 1] = dwa_of_mul(c0r, fy[c]);
-    }
-    dwa_mul(h[0], cz, fx[0]); dwa_mul(h[0], cr, fx[1]); dwa_sub(h[0], ci, fy[1]);
-    dwa_mul(h[1], cz, fy[0]); dwa_mul(h[1], cr, fy[1]); dwa_mul(h[1], ci, fx[1]);
-    dwa_mul(h[2], cr, fx[0]); dwa_mul(h[2], ci, fy[0]); dwa_mul(h[2], cr, fx[2]); dwa_sub(h[2], ci, fy[2]);
-    dwa_mul(h[3], cr, fy[0]); dwa_sub(h[3], ci, fx[0]); dwa_mul(h[3], cr, fy[2]); dwa_mul(h[3], ci, fx[2]);
-    dwa_mul(h[4], cr, fx[1]); dwa_mul(h[4], ci, fy[1]); dwa_sub(h[4], cz, fx[2]);
-    dwa_mul(h[5], cr, fy[1]); dwa_sub(h[5], ci, fx[1]); dwa_sub(h[5], cz, fy[2]);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      dwa_add(h[2 * c], hx[c].hi, hx[c].lo);
-      dwa_add(h[2 * c + 1], hy[c].hi, hy[c].lo);
+    for (int c = 0; c < 3; ++c)
       A.hphi[at + c * npts] = make_double2(dw_to_double(h[2 * c]), dw_to_double(h[2 * c + 1]));
-    }
-    dwa_sqd(acc[1], rho);
-    dwa_mul(acc[2], DF{ar.hi + ar.hi, ar.lo + ar.lo}, ar);
-    dwa_mul(acc[2], DF{ai.hi + ai.hi, ai.lo + ai.lo}, ai);
-    dwa_sqd(acc[2], Fz);
     const int row = (int)(off >> Lx);
     const float V = trap_value<float>(A.trap, A.g, (int)off & (nx - 1), row & (ny - 1), row >> Ly, off);
     const float rf = mf[0] + mf[1] + mf[2];
@@ -300,7 +249,7 @@ __global__ void __launch_bounds__(kHyThreads, kHyBlocksPerSM) k_hy_upd(HyArgs A)
   }
   DF all[12];
 #pragma unroll
-  for (int k = 0; k < 6; ++k) { all[k] = dwa_value(acc[k]); all[6 + k] = DF{acc32[k], 0.0f}; }
+  for (int k = 0; k < 6; ++k) { all[k] = acc[k]; all[6 + k] = DF{acc32[k], 0.0f}; }
   double v[12];
   block_reduce_dw<12>(all, v, scratch);
   const int slots[12] = {SL_Q, SL_RHO2, SL_F2, SL_M0, SL_M1, SL_M2, SL_V0, SL_V1, SL_V2, SL_C0, SL_C1, SL_C2};
