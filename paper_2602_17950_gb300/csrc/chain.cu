@@ -21,6 +21,7 @@
 #include <mutex>
 
 #include "gpsoc_internal.cuh"
+#include "hypoint.cuh"
 #include "scalar.cuh"
 #include "fft.cuh"
 
@@ -390,7 +391,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
 
   // ROW_INV_H / ROW_INV_P / ROW_INV_LIN: lin = F_x^-1(T')/npts - Omega x F_x^-1(G)/npts + V u
   const W Omn = Om * inv_n;
-  DF rphi{0.0f, 0.0f}, pp{0.0f, 0.0f};   // ROW_INV_P_HY: Re<P, Phi> against the FP64 Phi and ||P||^2 in double words
+  double rphi = 0.0, pp = 0.0;           // ROW_INV_P_HY: Re<P, Phi> against the FP64 Phi and ||P||^2
   W acc[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) acc[k] = (W)0;
@@ -402,7 +403,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
     const int row = row0 + r;
     C u[3];  // Phi for ROW_INV_H, P for ROW_INV_P / ROW_INV_LIN
     C f[3], h[3];
-    C fl[3];
+    double2 f64[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       u[c] = A.in2[at + c * npts];
@@ -410,7 +411,7 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
         f[c] = A.in3[at + c * npts];
         h[c] = A.in4[at + c * npts];
       }
-      if (MODE == ROW_INV_P_HY) fl[c] = A.philo[at + c * npts];
+      if (MODE == ROW_INV_P_HY) f64[c] = A.phi64[at + c * npts];
     }
     const W ox = Omn * coord<W>(A.g, 0, j);
     const W V = trap_value<W>(A.trap, A.g, j, row & (ny - 1), row >> Ly, at - (long long)s * 3 * npts);
@@ -457,16 +458,11 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
       acc[2] += (W)2 * (ax * ax + ay * ay) + Fz * Fz;
     } else {  // ROW_INV_P: step-model reductions (Eqs. an, bn and the sin/cos form of E(theta))
       if constexpr (MODE == ROW_INV_P_HY) {
-        // H_lin P kept for the update of H_lin Phi by linearity; the radial part of P (P's FP32
-        // values against Phi's double words, as the opening pass left them) and ||P||^2 to double-word accuracy for the exact tangent
-        // correction and the normalisation of the step
+        // H_lin P kept for the update of H_lin Phi by linearity; the radial part of P and ||P||^2 in FP64
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           A.out0[at + c * npts] = mk<C>(lin_r[c], lin_i[c]);
-          dwa_mulf(rphi, DF{f[c].x, fl[c].x}, u[c].x);
-          dwa_mulf(rphi, DF{f[c].y, fl[c].y}, u[c].y);
-          dwa_sq(pp, u[c].x);
-          dwa_sq(pp, u[c].y);
+          hy_radial(rphi, pp, f64[c].x, f64[c].y, u[c].x, u[c].y);
         }
       }
       W mx_[3], mf[3], mp[3];   // Re(f conj(u)), |f|^2, |u|^2 per component
@@ -503,7 +499,6 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
     }
   }
   if (MODE == ROW_INV_LIN) return;
-  const bool mx[14] = {};
   if (MODE == ROW_INV_H) {
     const bool mx12[12] = {};
     const int slots[12] = {SL_Q, SL_RHO2, SL_F2, SL_V0, SL_V1, SL_V2, SL_C0, SL_C1, SL_C2, SL_M0, SL_M1, SL_M2};
@@ -513,13 +508,9 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
     const int slots[14] = {SL_HPP, SL_HPHIP, SL_IFR, SL_IFP, SL_IRR, SL_IRP, SL_IPP,
                            SL_JFR, SL_JFP, SL_JRR, SL_JRP, SL_JPP, SL_RPHI, SL_P2};
     if constexpr (MODE == ROW_INV_P_HY) {
-      DF all[14];
-#pragma unroll
-      for (int k = 0; k < 12; ++k) all[k] = DF{acc[k], 0.0f};
-      all[12] = dwa_value(rphi);
-      all[13] = dwa_value(pp);
+      const bool mx[14] = {};
       double v[14];
-      block_reduce_dw<14>(all, v, red);
+      block_reduce_df_fp64<12>(acc, rphi, pp, v, red);
       put_partials<14>(A.part, sslot, A.pmax, rb, slots, v, mx, true);
       group_sums<DF, 14>(A.part + sslot * A.pmax, A.pmax, slots, rb, bps, gcnt, tail);
     } else {

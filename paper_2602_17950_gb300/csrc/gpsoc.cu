@@ -572,7 +572,6 @@ HyArgs hy_args(gpsoc_problem* p, int level, const Geo& g, const ScalarCtx& sc, i
   h.p = p->b32.P[(parity & 1) ^ 1];   // direction of the previous iteration
   h.hlp = p->b32.HPhi;                // its H_lin P
   h.phi32 = p->b32.Phi;
-  h.philo = p->b32.D;                 // free in hybrid iterations
   h.gcnt = p->d_cnt + p->batch;
   h.gmax = p->gmax;
   h.hphi = p->b64.Z;                  // H(Phi): the FP64 Z buffer is free in hybrid iterations
@@ -698,7 +697,7 @@ gpsoc_status enqueue_iteration_hy(gpsoc_problem* p, int level, int parity, const
   ChainArgs<float> pi = a;
   pi.fuse = 1;
   pi.in0 = F.W; pi.in1 = F.G; pi.in2 = F.P[cur]; pi.in3 = F.Phi; pi.in4 = F.R[cur];
-  pi.philo = F.D; pi.out0 = F.HPhi; pi.out1 = nullptr;
+  pi.phi64 = D.Phi; pi.out0 = F.HPhi; pi.out1 = nullptr;
   RL<float>(p, ROW_INV_P_HY, pi);
   CK(cudaGetLastError());
   return GPSOC_OK;

@@ -192,7 +192,6 @@ struct ChainArgs {
   ScalarCtx sc;
   // GPSOC_HYBRID passes of an FP32 chain that also read the FP64 state
   const double2* phi64;   // Phi (FP64)
-  const C* philo;         // low words of Phi (the FP32 copy holds the high ones), for ROW_INV_P_HY
   const double2* hl64;    // H(Phi) (FP64), for ROW_FWD_PRE_HY
   // GPSOC_HYBRID, last column pass of the P chain: the spectrum of Phi (advanced by the
   // step applied this iteration when khat_upd is set) and of the previous P, both updated
@@ -415,6 +414,26 @@ __device__ __forceinline__ double block_max(double x, double* scratch) {
   return __longlong_as_double((long long)r);
 }
 
+// warp sums of KP double words by reduce-scatter: lane l has the total of value (its low log2 KP bits reversed) in x[0]
+template <int KP>
+__device__ __forceinline__ void warp_reduce_dw(DF (&x)[KP]) {
+  constexpr int LB = (KP == 2) ? 1 : (KP == 4) ? 2 : (KP == 8) ? 3 : 4;
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int st = 0; st < LB; ++st) {
+    const int ofs = 1 << st, half = (KP / 2) >> st;
+    const bool up = (lane & ofs) != 0;
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const DF keep = up ? x[i + half] : x[i];
+      const DF send = up ? x[i] : x[i + half];
+      x[i] = dw_add(keep, df_shfl_xor(send, ofs));
+    }
+  }
+#pragma unroll
+  for (int ofs = KP; ofs < 32; ofs <<= 1) x[0] = dw_add(x[0], df_shfl_xor(x[0], ofs));
+}
+
 // Block sums of double-float per-thread partials, same fixed order and same
 // reduce-scatter scheme as block_reduce, with the accurate double-word sum; the K
 // totals are rounded to FP64 once at the end.  scratch: >= 16 * (blockDim.x / 32) + 16
@@ -432,19 +451,7 @@ __device__ __forceinline__ void block_reduce_dw(const DF (&a)[K], double (&v)[K]
     x[k].hi = (k < K) ? a[k].hi : 0.0f;
     x[k].lo = (k < K) ? a[k].lo : 0.0f;
   }
-#pragma unroll
-  for (int st = 0; st < LB; ++st) {
-    const int ofs = 1 << st, half = (KP / 2) >> st;
-    const bool up = (lane & ofs) != 0;
-#pragma unroll
-    for (int i = 0; i < half; ++i) {
-      const DF keep = up ? x[i + half] : x[i];
-      const DF send = up ? x[i] : x[i + half];
-      x[i] = dw_add(keep, df_shfl_xor(send, ofs));
-    }
-  }
-#pragma unroll
-  for (int ofs = KP; ofs < 32; ofs <<= 1) x[0] = dw_add(x[0], df_shfl_xor(x[0], ofs));
+  warp_reduce_dw<KP>(x);
   int slot = 0;
 #pragma unroll
   for (int b = 0; b < LB; ++b) slot |= ((lane >> b) & 1) << (LB - 1 - b);
@@ -464,6 +471,46 @@ __device__ __forceinline__ void block_reduce_dw(const DF (&a)[K], double (&v)[K]
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < K; ++k) v[k] = res[k];
+}
+// The same for K <= 14 FP32 partials in double words and two FP64 ones in FP64 (v[K], v[K + 1]), in the same
+// two barriers; the FP64 sums of the warps are added by the second warp.
+template <int K>
+__device__ __forceinline__ void block_reduce_df_fp64(const float (&a)[K], double b0, double b1, double (&v)[K + 2],
+                                                     double* scratch) {
+  static_assert(K > 8 && K <= 14, "16 values a warp");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  __syncthreads();  // scratch may alias shared memory the caller used just before
+  double y = ((lane & 1) ? b1 : b0) + __shfl_xor_sync(0xffffffffu, (lane & 1) ? b0 : b1, 1);
+#pragma unroll
+  for (int ofs = 2; ofs < 32; ofs <<= 1) y += __shfl_xor_sync(0xffffffffu, y, ofs);
+  DF x[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) x[k] = DF{k < K ? a[k < K ? k : 0] : 0.0f, 0.0f};
+  warp_reduce_dw<16>(x);
+  int slot = 0;
+#pragma unroll
+  for (int b = 0; b < 4; ++b) slot |= ((lane >> b) & 1) << (3 - b);
+  float2* sc2 = reinterpret_cast<float2*>(scratch);
+  if (lane < 16 && slot < K) sc2[warp * 16 + slot] = make_float2(x[0].hi, x[0].lo);
+  if (lane < 2) scratch[warp * 16 + K + lane] = y;
+  __syncthreads();
+  double* res = scratch + 16 * nw;
+  if (threadIdx.x < K) {
+    const float2 f = sc2[threadIdx.x];
+    DF acc{f.x, f.y};
+    for (int w = 1; w < nw; ++w) {
+      const float2 g = sc2[w * 16 + threadIdx.x];
+      acc = dw_add(acc, DF{g.x, g.y});
+    }
+    res[threadIdx.x] = (double)acc.hi + (double)acc.lo;
+  } else if (warp == 1 && lane < 2) {
+    double acc = scratch[K + lane];
+    for (int w = 1; w < nw; ++w) acc += scratch[w * 16 + K + lane];
+    res[K + lane] = acc;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < K + 2; ++k) v[k] = res[k];
 }
 // the same for FP32 per-thread partials
 template <int K>
@@ -539,7 +586,7 @@ enum RowMode {
   ROW_FWD_PRE_HY,      // FP32 pass of GPSOC_HYBRID: r = H Phi - mu Phi in FP64 from phi64 and H(Phi)
                        // (hl64) -> out1 (FP32); out0 = F_x(P_V^{1/2} r); reduce max|r|
   ROW_INV_P_HY         // FP32 pass of GPSOC_HYBRID: as ROW_INV_P with in4 = r (slot HPHIP = Re<r, P>),
-                       // out0 = H_lin P, and the step integrals with Phi = FP32 copy + low words
+                       // out0 = H_lin P; Re<P, Phi> against the FP64 Phi and ||P||^2 are FP64 sums
 };
 enum ColMode {
   COL_FWD = 0,         // out0 = F_axis(in0)

@@ -77,8 +77,7 @@ struct HyArgs {
   double2* hl;           // H_lin Phi (FP64), updated in place
   const float2* p;       // the pending direction P (FP32)
   const float2* hlp;     // H_lin P (FP32)
-  float2* phi32;         // FP32 copy of Phi for the FP32 passes: the high words of its double words
-  float2* philo;         // the low words
+  float2* phi32;         // FP32 copy of Phi for the FP32 passes
   unsigned* gcnt; int gmax;   // group arrival counters (group_sums)
   double2* hphi;         // H(Phi) = H_lin Phi + nonlinear terms (FP64), written by HY_REDUCE
   long long npts;

@@ -219,7 +219,6 @@ __global__ void __launch_bounds__(kHyThreads, kHyBlocksPerSM) k_hy_upd(HyArgs A)
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       A.phi32[at + c * npts] = make_float2(fx[c].hi, fy[c].hi);
-      A.philo[at + c * npts] = make_float2(fx[c].lo, fy[c].lo);
       mf[c] = fx[c].hi * fx[c].hi + fy[c].hi * fy[c].hi;   // the alpha pieces (FP32)
     }
     DF h[6];

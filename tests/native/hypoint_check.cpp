@@ -138,3 +138,20 @@ extern "C" int hp_errors(int seed, int threads, int points, double* rms, double*
     }
   return COUNT;
 }
+
+// sums of a thread's direction p (pairs) against phi (pairs) by hy_radial, and their errors
+extern "C" void hp_radial(int n, const double* phi, const float* p, double* got, double* want, double* moduli) {
+  double r = 0.0, s = 0.0;
+  Q er = 0, es = 0, mr = 0;
+  for (int i = 0; i < n; ++i) {
+    hy_radial(r, s, phi[2 * i], phi[2 * i + 1], p[2 * i], p[2 * i + 1]);
+    for (int k = 2 * i; k < 2 * i + 2; ++k) {
+      er += (Q)phi[k] * p[k];
+      mr += mod((Q)phi[k] * p[k]);
+      es += (Q)p[k] * p[k];
+    }
+  }
+  got[0] = r; got[1] = s;
+  want[0] = (double)(r - er); want[1] = (double)(s - es);
+  moduli[0] = (double)mr; moduli[1] = (double)es;
+}

@@ -32,3 +32,15 @@ def test_error_no_larger_than_term_by_term(lib, threads, points):
         # products within 7 u^2, a sum's rounding within 3 u^2, five levels of them at most, of values that are themselves
         # products of such (H(Phi), rho^2, |F|^2: three factors)
         assert most[0, k] <= 3 * (7 + 5 * 3), (name, most[:, k])
+
+
+@pytest.mark.parametrize("n", [1, 3, 24, 96])
+def test_radial_part_and_norm_are_fp64_sums(lib, n):
+    """FP64 products and sums: of the 2n terms each is rounded, and each sum of at most their moduli, 2^-53 each."""
+    rng = np.random.default_rng(n)
+    for _ in range(200):
+        phi = rng.normal(size=2 * n) * np.exp(-4 * rng.uniform())
+        p = (rng.normal(size=2 * n) * np.exp(-8 * rng.uniform())).astype(np.float32)
+        got, err, mod = np.zeros(2), np.zeros(2), np.zeros(2)
+        lib.hp_radial(n, *(C.c_void_p(a.ctypes.data) for a in (phi, p, got, err, mod)))
+        assert np.all(np.abs(err) <= (2 * n + 1) * 2.0 ** -53 * mod)
