@@ -250,28 +250,25 @@ __device__ __forceinline__ void row_pass(const ChainArgs<T>& A, int R, int ept) 
       } else if (MODE == ROW_FWD_PRE_HY) {
         // GPSOC_HYBRID: r = H Phi - mu Phi in FP64 from the FP64 state and H(Phi) (the residual
         // keeps FP64 accuracy: one fused multiply-add each), stored as FP32; the preconditioner's
-        // transforms then run on P_V^{1/2} r in FP32, P_V from FP32 values as in the pass that
-        // closes them.  6 FP64 instructions a point (22 with rho and the conversions on that pipe,
-        // which bound the pass: 308k of its 397k cycles at 64 x 256^2)
+        // transforms then run on P_V^{1/2} r in FP32, P_V from the FP64 state's density. max |r| is
+        // that of the FP64 r. 6 FP64 instructions a point (22 with the density and the conversions on that
+        // pipe, which bound the pass: 308k of its 397k cycles at 64 x 256^2)
         double2 f[3], h[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           f[c] = A.phi64[at + c * npts];
           h[c] = A.hl64[at + c * npts];
         }
-        W rho = (W)0;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const W fx = narrow_f(f[c].x), fy = narrow_f(f[c].y);
-          rho += fx * fx + fy * fy;
-        }
+        const long long pt = at - (long long)s * 3 * npts;
+        const W rho = A.rho32[(long long)s * npts + pt];
         const int row = row0 + r;
-        const W V = trap_value<W>(A.trap, A.g, j, row & (ny - 1), row >> Ly, at - (long long)s * 3 * npts);
+        const W V = trap_value<W>(A.trap, A.g, j, row & (ny - 1), row >> Ly, pt);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          const C rc = mk<C>(narrow_f(h[c].x - mu64 * f[c].x), narrow_f(h[c].y - mu64 * f[c].y));
+          const DF rx = dw_of(h[c].x - mu64 * f[c].x), ry = dw_of(h[c].y - mu64 * f[c].y);
+          const C rc = mk<C>(rx.hi, ry.hi);
           A.out1[at + c * npts] = rc;
-          acc[0] = max_pos(acc[0], rc.x * rc.x + rc.y * rc.y);
+          acc[0] = max_pos(acc[0], hy_square(rx, ry));
           const W den = max_pos(al[c] + (V + c0 * rho), (W)1e-12 * al[c]);
           const W sc = use_pv ? rsqrt_w(den) : (W)1;
           buf0[c * CP + pos] = mk<C>(rc.x * sc, rc.y * sc);

@@ -193,6 +193,7 @@ struct ChainArgs {
   // GPSOC_HYBRID passes of an FP32 chain that also read the FP64 state
   const double2* phi64;   // Phi (FP64)
   const double2* hl64;    // H(Phi) (FP64), for ROW_FWD_PRE_HY
+  const float* rho32;     // density of the FP64 Phi, for ROW_FWD_PRE_HY
   // GPSOC_HYBRID, last column pass of the P chain: the spectrum of Phi (advanced by the
   // step applied this iteration when khat_upd is set) and of the previous P, both updated
   // in place, for the exact per-component kinetic sums of alpha

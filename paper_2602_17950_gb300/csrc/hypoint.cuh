@@ -88,6 +88,11 @@ GPSOC_DW void hy_sums(DF (&acc)[6], const HyPoint& p, const DF (&fx)[3], const D
   for (int c = 0; c < 3; ++c) acc[3 + c] = dw_add(acc[3 + c], p.m[c]);
 }
 
+// |r|^2 of an FP64 residual given as double words, in FP32: the two products' roundings, u each
+GPSOC_DW float hy_square(DF x, DF y) {
+  return rn_fma(x.hi, x.hi, rn_fma(y.hi, y.hi, rn_fma(x.hi + x.hi, x.lo, rn_mul(y.hi + y.hi, y.lo))));
+}
+
 // a value's terms of the radial part Re<P, Phi> of the direction and of ||P||^2 (row_inv_p_hy): FP64 sums of an FP32
 // direction against the FP64 Phi, for the exact tangent correction and the normalisation of the step.  As double words
 // they made the totals' error two to five times as large for a 64 x 256^2 solve of 24.2 ms instead of 24.9

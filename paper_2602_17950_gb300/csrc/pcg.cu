@@ -215,6 +215,7 @@ __global__ void __launch_bounds__(kHyThreads, kHyBlocksPerSM) k_hy_upd(HyArgs A)
     // H(Phi) and the sums of the energy (Eq. energy) and of alpha_l (Eq. PreCnstAlpha)
     const HyPoint pt = hy_point(fx, fy);
     hy_sums(acc, pt, fx, fy, hx, hy);
+    A.rho32[(long long)s * npts + off] = pt.rho.hi;
     float mf[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {

@@ -155,3 +155,23 @@ extern "C" void hp_radial(int n, const double* phi, const float* p, double* got,
   want[0] = (double)(r - er); want[1] = (double)(s - es);
   moduli[0] = (double)mr; moduli[1] = (double)es;
 }
+
+// largest errors in u of |r|^2 by hy_square and of the density's FP32 value, over n random residuals and points
+extern "C" void hp_fp32(int seed, int n, double* most) {
+  std::mt19937_64 gen(seed);
+  std::normal_distribution<double> N;
+  std::uniform_real_distribution<double> U(0, 1);
+  most[0] = most[1] = 0.0;
+  for (int i = 0; i < n; ++i) {
+    const double scale = exp(-20 * U(gen));
+    DF f[6], fx[3], fy[3];
+    for (int k = 0; k < 6; ++k) f[k] = dw_of(scale * N(gen));
+    for (int c = 0; c < 3; ++c) { fx[c] = f[2 * c]; fy[c] = f[2 * c + 1]; }
+    const double x = scale * N(gen), y = scale * N(gen);
+    const Q r2 = (Q)x * x + (Q)y * y, got = hy_square(dw_of(x), dw_of(y));
+    Q rho = 0;
+    for (int k = 0; k < 6; ++k) rho += q(f[k]) * q(f[k]);
+    const double e[2] = {(double)(mod(got - r2) / r2), (double)(mod(hy_point(fx, fy).rho.hi - rho) / rho)};
+    for (int k = 0; k < 2; ++k) most[k] = e[k] * 16777216.0 > most[k] ? e[k] * 16777216.0 : most[k];
+  }
+}

@@ -44,3 +44,12 @@ def test_radial_part_and_norm_are_fp64_sums(lib, n):
         got, err, mod = np.zeros(2), np.zeros(2), np.zeros(2)
         lib.hp_radial(n, *(C.c_void_p(a.ctypes.data) for a in (phi, p, got, err, mod)))
         assert np.all(np.abs(err) <= (2 * n + 1) * 2.0 ** -53 * mod)
+
+
+def test_fp32_values_are_of_the_fp64_state(lib):
+    """|r|^2 of the FP64 residual: two roundings of u each, and u times the cross terms (2u of it each) and the low words'
+    squares; the density is a double word's high word: half an ulp (u) and what the low word is off by, some u^2."""
+    most = np.zeros(2)
+    lib.hp_fp32(5, 200000, C.c_void_p(most.ctypes.data))
+    u = 2.0 ** -24
+    assert most[0] <= 2 + 8 * u and most[1] <= 1 + 64 * u
