@@ -90,16 +90,11 @@ __device__ __forceinline__ void spin_a(C1 p1, C2 p0, C3 pm, W& ar, W& ai) {
   ai = (W)p0.x * (W)p1.y - (W)p0.y * (W)p1.x + (W)pm.x * (W)p0.y - (W)pm.y * (W)p0.x;
 }
 
-// 1/sqrt(x), x > 0.  FP64: the FP32 value as a start (the integer pipes convert), then
-// y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2, |e| < 2^-20, to e^3: 5 FP64 instructions against 9 of the
+// 1/sqrt(x), x > 0.  FP64: from the FP32 value (the integer pipes convert), 4 FP64 instructions against 9 of the
 // library's; outside the FP32 range the library
 __device__ __forceinline__ float rsqrt_w(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_w(double x) {
-  const int h = __double2hiint(x);
-  if (h < 0x39000000 || h > 0x46f00000) return rsqrt(x);   // below 2^-111, above 2^112, or negative
-  const double y = widen_f(rsqrtf(narrow_f(x)));
-  const double e = 1.0 - (x * y) * y;
-  return y + y * (e * (0.375 * e + 0.5));
+  return rsqrt_in_range(x) ? rsqrt_refine(x, widen_f(rsqrtf(narrow_f(x)))) : rsqrt(x);
 }
 // larger of two values, the second positive: their bits are ordered alike (and a negative or
 // smaller first one is below), without the FP64 pipe

@@ -15,6 +15,7 @@
 
 #include "../../include/gpsoc.h"
 #include "dword.cuh"
+#include "fp64math.cuh"
 
 namespace gpsoc {
 

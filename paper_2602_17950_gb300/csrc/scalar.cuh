@@ -374,27 +374,14 @@ __device__ __forceinline__ double energy_change(const SolveState& S, double thet
   return energy_change_sc(S, sn, cs, rsqrt(S.P2));
 }
 
-// sine and cosine of the step's angle, by a whole warp: their Taylor sums (to x^19 and x^18, below
-// 2^-56 of the value for x <= 0.8) on the odd and the even lanes, 12 FP64 instructions instead of the
-// library's 27; larger angles by the library
+// sine and cosine of the step's angle, by a whole warp: their Taylor sums on the odd and the even lanes,
+// 12 FP64 instructions instead of the library's 27; larger angles (and negative ones, NaN) by the library
 __device__ __forceinline__ void sincos_warp(double x, double& sn, double& cs) {
-  if (!(__double2hiint(x) < 0x3fe99999 && __double_as_longlong(x) >= 0)) {   // x >= 0.8 (or negative)
+  if (!taylor_in_range(x)) {
     sincos(x, &sn, &cs);
     return;
   }
-  const bool odd = threadIdx.x & 1;
-  const double x2 = x * x;
-  double r = odd ? -1.0 / 121645100408832000.0 : -1.0 / 6402373705728000.0;    // 1/19!, 1/18!
-  r = r * x2 + (odd ? 1.0 / 355687428096000.0 : 1.0 / 20922789888000.0);       // 1/17!, 1/16!
-  r = r * x2 + (odd ? -1.0 / 1307674368000.0 : -1.0 / 87178291200.0);
-  r = r * x2 + (odd ? 1.0 / 6227020800.0 : 1.0 / 479001600.0);
-  r = r * x2 + (odd ? -1.0 / 39916800.0 : -1.0 / 3628800.0);
-  r = r * x2 + (odd ? 1.0 / 362880.0 : 1.0 / 40320.0);
-  r = r * x2 + (odd ? -1.0 / 5040.0 : -1.0 / 720.0);
-  r = r * x2 + (odd ? 1.0 / 120.0 : 1.0 / 24.0);
-  r = r * x2 + (odd ? -1.0 / 6.0 : -0.5);
-  const double f = odd ? x : 1.0;
-  r = (r * x2) * f + f;
+  const double r = taylor_sincos(x, threadIdx.x & 1);
   cs = __shfl_sync(0xffffffffu, r, 0);
   sn = __shfl_sync(0xffffffffu, r, 1);
 }
@@ -478,9 +465,7 @@ __device__ __forceinline__ double step_sums(const ScalarCtx& X, int s, const dou
   // which is tangent to the sphere whatever the rounding of P (an FP32 direction carries a
   // radial part of relative size 1e-7).  Every sum transforms exactly: R -> R - a rho_Phi,
   // rho_P -> rho_P - 2a R + a^2 rho_Phi, and the same for the spin vectors.
-  // ||Phi||^2 is 1 up to rounding, where 1/M = 2 - M
-  const double d = 1.0 - M;
-  const double a = (__double2hiint(d) & 0x7fffffff) < 0x3e500000 /* |d| < 2^-26 */ ? RPhi + d * RPhi : RPhi / M;
+  const double a = divide_near_one(RPhi, M);   // ||Phi||^2 is 1 up to rounding
   const double Z1 = K1 - a * K0, Z2 = K2 - a * (K1 + Z1);
   const double q = K3 - a * K1, Z3 = q - a * Z1;
   const double w = K4 - a * (K3 + q), Z4 = w - a * Z2;
@@ -557,10 +542,9 @@ __device__ __forceinline__ void step_decide(const ScalarCtx& X, SolveState& S, d
   const double sp = sn * inv;
   const double M = S.mass[0] + S.mass[1] + S.mass[2];
   // Phi' = (cos t Phi + sin t P_t/|P_t|)/norm with P_t = P - a Phi tangent: |.|^2 = c^2 M + s'^2 |P_t|^2,
-  // which is 1 up to rounding: 1/sqrt(1 + d) = 1 - d/2 + 3 d^2/8 - ... to d^2
+  // which is 1 up to rounding
   const double d = (cs * cs * M + sp * sp * S.P2) - 1.0;
-  const double g = (__double2hiint(d) & 0x7fffffff) < 0x3ee00000 /* |d| < 2^-17 */ ? 1.0 + d * (0.375 * d - 0.5)
-                                                                                 : rsqrt(1.0 + d);
+  const double g = rsqrt1_in_range(d) ? rsqrt1(d) : rsqrt(1.0 + d);
   const double uc = cs - sp * S.acorr;
   __syncwarp();
   if (one) {
