@@ -86,6 +86,12 @@ __global__ void k_setup(SolveState* st, unsigned* cnt, PhysDev* phys, SetupParam
   phys[first + k] = q.p[k];
 }
 
+// What a state and a point of an axis count in the budget.  They are the sizes of an earlier layout (a larger state, a
+// twiddle table per axis) and stay what they were, so that a request that fitted still fits; the arrival
+// counters lie in the axes' share.
+constexpr size_t kStateBudget = 488, kAxisBudget = 16;
+static_assert(sizeof(SolveState) <= kStateBudget, "the budget of a state is part of the call's limit");
+
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 int ilog2i(int n) { int l = 0; while ((1 << l) < n) ++l; return l; }
@@ -130,14 +136,19 @@ extern "C" gpsoc_status gpsoc_apply_h_noalloc(const gpsoc_grid* grid, const gpso
   size_t off = 0;
   const size_t o_arr = off; off += align256(4 * arr);
   const size_t o_part = off; off += align256(sizeof(double) * (size_t)batch * NSLOT * pmax);
-  // 56 bytes a state and a table per axis are spare: part of the budget callers know
-  const size_t o_st = off; off += align256((sizeof(SolveState) + 56) * batch);
+  const size_t o_st = off; off += align256(kStateBudget * batch);
   const size_t o_ph = off; off += align256(sizeof(PhysDev) * batch);
   const size_t o_cnt = off;
-  for (int i = 0; i < g.d; ++i) off += align256(sizeof(double2) * g.n[i]);
+  for (int i = 0; i < g.d; ++i) off += align256(kAxisBudget * g.n[i]);
   const size_t o_obs = off; off += align256(sizeof(double) * 9 * batch);
-  if (off > kNoAllocScratchBytes) {
-    return GPSOC_EBUDGET;
+  // a group counter per 64 blocks: 4 (1 + pmax / 64) bytes a solve of the axes' share and the observables' 72
+  const int gmax = (pmax + 63) / 64;
+  if (off > kNoAllocScratchBytes || sizeof(unsigned) * (size_t)batch * (1 + gmax) > off - o_cnt) return GPSOC_EBUDGET;
+  // every check before the first launch: a call that returns an error leaves nothing running
+  for (int k = 0; k < batch; ++k) {
+    const gpsoc_params& r = params[k];
+    if (!std::isfinite(r.Omega) || !std::isfinite(r.gamma) || !std::isfinite(r.beta0) || !std::isfinite(r.beta1))
+      return GPSOC_EINVAL;
   }
   unsigned char* base = nullptr;
   cudaError_t e = scratch_address(&base);
@@ -151,19 +162,14 @@ extern "C" gpsoc_status gpsoc_apply_h_noalloc(const gpsoc_grid* grid, const gpso
   SolveState* sst = (SolveState*)(base + o_st);
   PhysDev* ph = (PhysDev*)(base + o_ph);
   double* dobs = (double*)(base + o_obs);
-  // arrival counters of every solve's blocks and groups of 64 blocks: in the spare tables and, where many small
+  // arrival counters of every solve's blocks and groups of 64 blocks: in the axes' share and, where many small
   // solves need it, on into the place of the gathered observables, which are written after the last arrival
   unsigned* cnt = (unsigned*)(base + o_cnt);
-  const int gmax = (pmax + 63) / 64;
-  if (sizeof(unsigned) * (size_t)batch * (1 + gmax) > off - o_cnt) return GPSOC_EBUDGET;   // 4 (1 + pmax / 64) of 72+ bytes
   for (int b0 = 0; b0 < batch; b0 += kSetup) {
     SetupParams q;
     const int nb = std::min(kSetup, batch - b0);
     for (int k = 0; k < nb; ++k) {
       const gpsoc_params& r = params[b0 + k];
-      if (!std::isfinite(r.Omega) || !std::isfinite(r.gamma) || !std::isfinite(r.beta0) || !std::isfinite(r.beta1)) {
-        return GPSOC_EINVAL;
-      }
       q.p[k] = make_phys(r.Omega, r.gamma, r.beta0, r.beta1);
     }
     k_setup<<<1, kSetup, 0, st>>>(sst, cnt, ph, q, b0, nb, 1 + gmax);
