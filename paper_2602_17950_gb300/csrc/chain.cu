@@ -932,9 +932,7 @@ template <class T>
 static size_t row_smem(const Geo& g, int mode, int nsolve) {
   using C = cx_t<T>;
   const int R = row_rows_per_block<T>(g, nsolve);
-  const int per = R * g.n[0];
   const bool two = (mode == ROW_INV_H || mode == ROW_INV_P || mode == ROW_INV_LIN || mode == ROW_INV_P_HY);
-  (void)per;
   const int CP = R * fft_padded_len<C>(g.n[0]);
   return sizeof(C) * (fft_padded_len<C>(g.n[0]) + 3 * CP * (two ? 2 : 1)) + kRedDoubles * sizeof(double);
 }

@@ -136,7 +136,6 @@ GPSOC_DW DF dw_neg(DF a) {
   r.lo = -a.lo;
   return r;
 }
-GPSOC_DW DF dw_sub(DF a, DF b) { return dw_add(a, dw_neg(b)); }
 GPSOC_DW DF dw_mul(DF a, DF b) {
   const float ch = rn_mul(a.hi, b.hi);
   const float cl = rn_fma(a.hi, b.hi, -ch);                       // TwoProd: a.hi b.hi = ch + cl

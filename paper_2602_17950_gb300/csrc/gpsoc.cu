@@ -103,9 +103,9 @@ const char* row_name(int m) {
   return (m >= 0 && m < (int)(sizeof(n) / sizeof(n[0]))) ? n[m] : "row_?";
 }
 const char* col_name(int m, int axis) {
-  static const char* n[2][7] = {{"coly_fwd", "coly_inv", "coly_mid_h", "coly_mid_pre", "coly_ymid_h", "coly_yinv_h", "coly_kin"},
-                                {"colz_fwd", "colz_inv", "colz_mid_h", "colz_mid_pre", "colz_ymid_h", "colz_yinv_h", "colz_kin"}};
-  return (m >= 0 && m < 7) ? n[axis == 2 ? 1 : 0][m] : "col_?";
+  static const char* n[2][6] = {{"coly_fwd", "coly_inv", "coly_mid_h", "coly_mid_pre", "coly_ymid_h", "coly_yinv_h"},
+                                {"colz_fwd", "colz_inv", "colz_mid_h", "colz_mid_pre", "colz_ymid_h", "colz_yinv_h"}};
+  return (m >= 0 && m < 6) ? n[axis == 2 ? 1 : 0][m] : "col_?";
 }
 const char* scalar_name(int ph) {
   static const char* n[] = {"sc_init", "sc_obs", "sc_clear", "sc_norm", "sc_model", "sc_kin"};

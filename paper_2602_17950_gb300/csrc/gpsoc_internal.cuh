@@ -597,7 +597,6 @@ enum ColMode {
   COL_MID_PRE,         // last axis, preconditioner: out0 = F^-1[F in0 / (alpha_l + |k|^2/2)]
   COL_YMID_H,          // 2D y pass of the H chain: out0 = T', out1 = G
   COL_YINV_H,          // 3D y inverse pass of the H chain: in0 = C, in1 = A -> out0 = T', out1 = G
-  COL_MID_KIN          // last axis: reduce kinetic per component only (no output)
 };
 
 template <class T>
