@@ -133,11 +133,12 @@ KERNEL_WORK = {
 # Hybrid iteration (FP64 state, FP32 directions): algorithmic bytes per grid point and
 # component of each pass (FP64 complex 16 B, FP32 complex 8 B; every array read or
 # written once).  hy_upd: R Phi, H_lin Phi (FP64), P, H_lin P (FP32); W Phi, H_lin Phi,
-# H(Phi) (FP64), FP32 Phi.  row_fwd_pre_hy: R Phi, H(Phi); W r, F_x(P_V^1/2 r).
+# H(Phi) (FP64), FP32 Phi and the density (4 B a point).  row_fwd_pre_hy: R Phi, H(Phi), the density; W r,
+# F_x(P_V^1/2 r).
 # row_inv_pre: R spectrum, FP32 Phi, r, r_prev, P_prev; W z.  coly_ymid_h in the hybrid P
 # chain also reads and writes the spectra of Phi and P.  row_inv_p_hy: R T', G, P, FP32
 # Phi, r, FP64 Phi; W H_lin P.
-HYBRID_BYTES = {"hy_upd": 104, "row_fwd_pre_hy": 48, "coly_mid_pre": 16, "row_inv_pre": 48,
+HYBRID_BYTES = {"hy_upd": 104 + 4 / 3, "row_fwd_pre_hy": 48 + 4 / 3, "coly_mid_pre": 16, "row_inv_pre": 48,
                 "row_fwd_proj": 40, "coly_ymid_h": 56, "row_inv_p_hy": 64}
 
 

@@ -144,6 +144,7 @@ __global__ void k_elem(ElemArgs<T> A) {
 // sub-partition; FP64 instructions remain only to split the loaded values and to round
 // the stored ones.  The alpha_l pieces V |phi_l|^2 and rho |phi_l|^2, which only shift
 // the preconditioner, are FP32 products; max |Phi' - Phi|^2 is taken from the high words.
+// The arithmetic is hypoint.cuh's.  The density goes to the residual pass as FP32.
 // The block sums are double words, stored as double-word partials for the observables
 // step (grid sums on the FP32 pipes, totals rounded to FP64).
 constexpr int kHyThreads = 256, kHyBlocksPerSM = 2;
