@@ -54,8 +54,8 @@ enum { GPSOC_TRAP_HARMONIC = 0, GPSOC_TRAP_HARMONIC_QUARTIC = 1, GPSOC_TRAP_USER
 /* Precision of a solve.  FP64: every array and operation in FP64.  MIXED: an FP32
  * phase per level (FP32 arrays, FP64 sums and step decisions) until the FP32
  * rounding floor, then FP64 iterations to the stopping rule.  HYBRID: after an
- * FP64 lead-in (hybrid_lead_res), FP64 wave function, residual, reductions and
- * step decisions, with H_lin Phi advanced by linearity from an FP32 H_lin P and
+ * FP64 lead-in (hybrid_lead_res), FP64 wave function, residual and step decisions
+ * (sums of the state in double words of two FP32, about 48 bits, or in FP64), with H_lin Phi advanced by linearity from an FP32 H_lin P and
  * recomputed in FP64 every hybrid_refresh iterations and before a residual is
  * accepted; the preconditioner's and the search direction's transforms run in
  * FP32.  HYBRID stops on the same FP64 rule as FP64 and reaches its fixed point. */
